@@ -44,7 +44,7 @@ struct gb_ctx {
     gbk::TaskList tasks;
     int wpb = 4;
     int tpt = 0;
-    int64_t total_tiles = 0;
+    int64_t total_cols = 0;
     std::string msg;
     cudaStream_t cs = nullptr;          // private stream for graph capture
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
@@ -110,49 +110,40 @@ cudaError_t zalloc(T** p, size_t n) {
     return cudaMemset(*p, 0, std::max<size_t>(n, 1) * sizeof(T));
 }
 
-// Cut the work of all replicas (super-rows of 64 atoms against 32-atom tiles
-// J >= 2K, replicas in order) into runs of `tpt` tiles, one warp task each.
+// Cut the work of replica r (row pairs of 128 atoms against 32-atom tiles
+// J >= 4P) into warp tasks of about `tpt` 64 x 32 blocks that stay within a
+// row pair.  The four columns on the diagonal hold the most close pairs: each
+// of their rows is a task of its own, as is each row of a small replica when
+// tpt is 1.
+void cut_replica(const gb_ctx* c, int r, int tpt, std::vector<int4>& out) {
+    const int nb = (int)((c->off_h[r + 1] - c->off_h[r] + 31) / 32);
+    const int cols = std::max(1, tpt / 2);
+    for (int P = 0; 4 * P < nb; ++P) {
+        const int rows_until = (tpt == 1 && nb <= gbk::SMALL_TILES) ? nb : std::min(nb, 4 * P + 4);
+        for (int J = 4 * P; J < rows_until; ++J) {
+            out.push_back(make_int4(r, 4 * P + 1, J, 1));
+            if (J >= 4 * P + 2) out.push_back(make_int4(r, 4 * P + 2, J, 1));
+        }
+        for (int J = std::max(rows_until, 4 * P + 4); J < nb; J += cols) out.push_back(make_int4(r, 4 * P + 3, J, std::min(cols, nb - J)));
+    }
+}
+
 int build_tasks_into(gb_ctx* c, int tpt, gbk::TaskList& out) {
     std::vector<int4> t;
-    t.reserve((size_t)(c->total_tiles / tpt + 1));
-    int64_t left_total = c->total_tiles;
-    int r = 0, K = 0, J = 0;
-    auto nb_of = [&](int rr) { return (int)((c->off_h[rr + 1] - c->off_h[rr] + 31) / 32); };
-    while (r < c->M && nb_of(r) == 0) ++r;
-    while (left_total > 0) {
-        const int cnt = (int)std::min<int64_t>(tpt, left_total);
-        t.push_back(make_int4(r, K, J, cnt));
-        left_total -= cnt;
-        int64_t k = cnt;
-        while (k > 0 && r < c->M) {
-            const int nb = nb_of(r);
-            const int rowleft = nb - J;
-            if (k < rowleft) {
-                J += (int)k;
-                k = 0;
-            } else {
-                k -= rowleft;
-                ++K;
-                if (K == (nb + 1) / 2) {
-                    ++r;
-                    while (r < c->M && nb_of(r) == 0) ++r;
-                    K = 0;
-                }
-                J = 2 * K;
-            }
-        }
-    }
-    // Costly blocks first: those at and next to a super-row's diagonal hold the
+    t.reserve((size_t)(2 * c->total_cols / tpt + 1));
+    for (int r = 0; r < c->M; ++r) cut_replica(c, r, tpt, t);
+    // Costly blocks first: those at and next to the diagonal hold the
     // chain's near pairs (closed forms, no far-block shortcut), so starting
     // them early leaves the cheap far blocks for the end of the pass, where
     // they even out the finishing times of the SMs.  Any order gives the same
     // fixed-point sums.
     std::stable_sort(t.begin(), t.end(), [](const int4& a, const int4& b) {
-        return a.z - 2 * a.y < b.z - 2 * b.y;
+        return a.z - (a.y & ~3) < b.z - (b.y & ~3);
     });
     if (out.d_tasks) cudaFree(out.d_tasks);
     out.d_tasks = nullptr;
     out.n_tasks = (int)t.size();
+    out.small = c->max_n <= 32 * gbk::SMALL_TILES;
     GB_CHECK(c, zalloc(&out.d_tasks, t.size()));
     if (!t.empty())
         GB_CHECK(c, cudaMemcpy(out.d_tasks, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice));
@@ -161,41 +152,29 @@ int build_tasks_into(gb_ctx* c, int tpt, gbk::TaskList& out) {
 
 int build_tasks(gb_ctx* c) { return build_tasks_into(c, c->tpt, c->tasks); }
 
-// Tables of the persistent MD kernel: per-replica pair tasks (runs of `tpt`
-// tiles that never leave their replica), item offsets and counts of the six
+// Tables of the persistent MD kernel: per-replica pair tasks (about `tpt`
+// blocks each), item offsets and counts of the six
 // phases.  The grid is sized to the resident capacity of the device.
 int setup_persist(gb_ctx* c) {
     int dev = 0, sms = 0, per_sm = 0;
     GB_CHECK(c, cudaGetDevice(&dev));
     GB_CHECK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     GB_CHECK(c, gbk::persist_occupancy(c->p.rep_k != 0.0f ? 1 : 0, &per_sm));
-    if (per_sm < 1 || c->total_tiles == 0) {
+    if (per_sm < 1 || c->total_cols == 0) {
         c->persist_grid = 0;
         return GB_OK;
     }
     c->persist_grid = sms * per_sm;
     const int64_t warps = (int64_t)c->persist_grid * 4;
     // about four pair items per resident warp and pass
-    const int tpt = (int)std::max<int64_t>(1, c->total_tiles / (4 * warps));
+    const int tpt = (int)std::max<int64_t>(1, 2 * c->total_cols / (4 * warps));
     const int M = c->M;
     std::vector<int4> t;
     std::vector<int> toff(M + 1, 0), cnt(6 * M, 0), poff(6 * (M + 1), 0);
     for (int r = 0; r < M; ++r) {
         const int64_t n = c->off_h[r + 1] - c->off_h[r];
-        const int nb = (int)((n + 31) / 32), nk = (nb + 1) / 2;
-        int64_t left = gbk::pair_units(n);
-        int K = 0, J = 0;
-        while (left > 0) {
-            const int run = (int)std::min<int64_t>(tpt, left);
-            t.push_back(make_int4(r, K, J, run));
-            left -= run;
-            int64_t k = run;
-            while (k > 0 && K < nk) {
-                const int rowleft = nb - J;
-                if (k < rowleft) { J += (int)k; k = 0; }
-                else { k -= rowleft; ++K; J = 2 * K; }
-            }
-        }
+        const int nb = (int)((n + 31) / 32);
+        cut_replica(c, r, tpt, t);
         toff[r + 1] = (int)t.size();
         const int tasks_r = toff[r + 1] - toff[r];
         const int per_phase[6] = {nb, tasks_r, nb, tasks_r, nb, tasks_r};
@@ -225,9 +204,9 @@ int default_tpt(const gb_ctx* c) {
     // a cutoff most blocks are skipped and the rest cluster along the diagonal,
     // so tasks eight times shorter even out the warps' work
     const int64_t slots = 152LL * 32 * 4;
-    int64_t t = (c->total_tiles + slots - 1) / slots;
+    int64_t t = (2 * c->total_cols + slots - 1) / slots;
     if (c->p.rgbmax > 0.0f || c->p.cut > 0.0f) t = (t + 7) / 8;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(t, 256));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(t, 64));
 }
 
 gbk::PairArgs pair_args(const gb_ctx* c, const float* xyzq, const float* rad) {
@@ -244,6 +223,7 @@ gbk::PairArgs pair_args(const gb_ctx* c, const float* xyzq, const float* rad) {
     a.kappa = c->p.kappa;
     a.rep_k = c->p.rep_k;
     a.rep_sigma = c->p.rep_sigma;
+    gbk::set_energy_factors(a, c->p);
     gbk::set_cutoffs(a, c->p);
     a.I_acc = c->I_acc;
     a.dR_acc = c->dR_acc;
@@ -388,7 +368,7 @@ extern "C" int gb_ctx_create(gb_ctx** out, int32_t n_rep, const int64_t* atom_of
     for (int r = 0; r < n_rep; ++r) {
         const int64_t n = atom_off[r + 1] - atom_off[r];
         c->max_n = (int32_t)std::max<int64_t>(c->max_n, n);
-        c->total_tiles += gbk::pair_units(n);
+        c->total_cols += gbk::pair_columns(n);
     }
     const size_t N = (size_t)c->N;
     cudaError_t e = cudaSuccess;
@@ -416,14 +396,14 @@ extern "C" int gb_ctx_create(gb_ctx** out, int32_t n_rep, const int64_t* atom_of
             e = cudaMemcpy(c->tile_off, toff.data(), sizeof(int) * (n_rep + 1), cudaMemcpyHostToDevice);
         step(zalloc(&c->boxes, 2 * (size_t)std::max(c->n_tiles32, 1)));
         if (params->rgbmax > 0.0f || params->cut > 0.0f) {
-            // every block of the batch may be in range: one task of one block each
+            // both rows of every column of the batch may be in range: one task each
             std::vector<int> woff(n_rep + 1, 0);
             for (int r = 0; r < n_rep; ++r) {
                 const int64_t nb = (atom_off[r + 1] - atom_off[r] + 31) / 32;
-                woff[r + 1] = woff[r] + (int)(((nb + 1) / 2) * ((nb + 31) / 32));
+                woff[r + 1] = woff[r] + (int)(((nb + 3) / 4) * ((nb + 31) / 32));
             }
             c->list_warps = woff[n_rep];
-            const size_t cap = (size_t)std::max<int64_t>(c->total_tiles, 1);
+            const size_t cap = (size_t)std::max<int64_t>(2 * c->total_cols, 1);
             if (params->rgbmax > 0.0f) step(zalloc(&c->list_b, cap));
             if (params->cut > 0.0f) step(zalloc(&c->list_e, cap));
             step(zalloc(&c->list_ctr, gbk::LIST_CTRS));
@@ -443,7 +423,8 @@ extern "C" int gb_ctx_create(gb_ctx** out, int32_t n_rep, const int64_t* atom_of
         return code;
     }
     c->tpt = default_tpt(c);
-    for (int k = 0; k < 3; ++k) c->tasks.cap[k] = 3;
+    c->wpb = c->max_n <= 32 * gbk::SMALL_TILES ? 2 : 4;
+    for (int k = 0; k < 3; ++k) c->tasks.cap[k] = c->list_ctr ? 3 : 1;
     int rc = build_tasks(c);
     if (rc == GB_OK) rc = setup_persist(c);
     if (rc != GB_OK) {

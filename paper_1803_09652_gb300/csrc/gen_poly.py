@@ -10,7 +10,12 @@ Both are fitted on [0, Y_MAX] by interpolation at Chebyshev nodes (a
 near-minimax fit), reference values from the series summed in FP64 to
 convergence, and emitted as monomial coefficients for Horner evaluation.
 A second, lower-degree pair (suffix "f") covers only the far field
-y <= Y_FAR, where fewer terms reach the same FP32 accuracy.
+y <= Y_FAR, where fewer terms reach the same FP32 accuracy, a third (suffix
+"n") y <= Y_NEAR.  Farther still the
+series needs three or four terms; those fits are emitted as coefficient lists
+(GB_G2, GB_G3, GB_H2, GB_H3) for blocks that evaluate them as polynomials in
+1/r^2 with the powers of s folded into per-atom coefficients, each with the
+largest y (GB_Y_G2 ...) for which the fit stays within 6e-8 of the series.
 
 With a Born-radius cutoff the integral of disjoint spheres is restricted to
 shells t in [L, U'] (L = r - s, U' = min(r + s, rc)).  With z = (U' - L)/U'
@@ -26,7 +31,10 @@ import os
 import numpy as np
 
 Y_MAX = 0.36     # x <= 0.6: every non-overlapping pair of the radius sets used here
+Y_NEAR = 0.20    # x <= 0.447: the pairs of near blocks that are not evaluated one by one
 Y_FAR = 0.10     # x <= 0.316: pairs more than ~3 screened radii apart
+# degree and range of the distant fits of g and h
+Y_DISTANT = {"g": ((3, 0.0250), (2, 0.0090)), "h": ((3, 0.0185), (2, 0.0060))}
 Z_J = 0.50       # z <= 1/2: restricted shells no wider than their inner radius
 Z_J2 = 0.75      # z <= 3/4: every pair of disjoint spheres of the radius sets used here
 
@@ -103,6 +111,24 @@ def emit(fh, name, deg, c, err, y_max, y_min=0.0):
     fh.write(f"__device__ __forceinline__ float2 gb_poly_{name}2(float2 y) {{\n    return {expr};\n}}\n")
 
 
+def distant_fits():
+    """(name, degree, y_max, FP32 coefficients, error) of the distant fits; the
+    error is that of the FP32 coefficients, evaluated in FP64."""
+    global Y_MAX
+    keep, out = Y_MAX, []
+    for name, f in (("g", g_exact), ("h", h_exact)):
+        for deg, y_max in Y_DISTANT[name]:
+            Y_MAX = y_max
+            c = fit(f, deg).astype(np.float32)
+            ys = np.linspace(0.0, y_max, 20001)
+            err = np.max(np.abs(np.polyval(c[::-1].astype(np.float64), ys) / f(ys) - 1.0))
+            if err > 6e-8:
+                raise RuntimeError(f"{name} degree {deg}: {err:.1e}")
+            out.append((name, deg, y_max, c, err))
+    Y_MAX = keep
+    return out
+
+
 def q_fit():
     zs = np.linspace(0.0, Z_J, 20001)
     for deg in range(2, 20):
@@ -133,6 +159,7 @@ def q2_fit():
 def main(out=None):
     full = best_fits(Y_MAX)
     far = best_fits(Y_FAR)
+    near = best_fits(Y_NEAR)
     qdeg, qc, qerr = q_fit()
     q2deg, q2c, q2err, z0 = q2_fit()
     here = os.path.dirname(os.path.abspath(__file__))
@@ -145,6 +172,14 @@ def main(out=None):
             emit(fh, name, deg, c, err, Y_MAX)
         for name, (deg, c, err) in far.items():
             emit(fh, name + "f", deg, c, err, Y_FAR)
+        fh.write(f"#define GB_POLY_YNEAR {Y_NEAR:.8f}f\n")
+        for name, (deg, c, err) in near.items():
+            emit(fh, name + "n", deg, c, err, Y_NEAR)
+        for name, deg, y_max, c, err in distant_fits():
+            key = f"{name.upper()}{deg}"
+            vals = ", ".join(f"{float(v):.9e}f" for v in c)
+            fh.write(f"/* {name}(y) on [0, {y_max:g}], degree {deg}, relative error of the coefficients {err:.2e} */\n")
+            fh.write(f"#define GB_Y_{key} {y_max:.8f}f\n#define GB_{key} {{{vals}}}\n")
         fh.write(f"#define GB_POLY_ZJ {Z_J:.8f}f\n")
         emit(fh, "q", qdeg, qc, qerr, Z_J)
         fh.write(f"#define GB_POLY_ZJ2 {Z_J2:.8f}f\n#define GB_POLY_ZMID {z0:.8f}f\n")
@@ -156,6 +191,8 @@ def main(out=None):
         print(name, deg, err)
     for name, (deg, c, err) in far.items():
         print(name + "f", deg, err)
+    for name, (deg, c, err) in near.items():
+        print(name + "n", deg, err)
 
 
 if __name__ == "__main__":

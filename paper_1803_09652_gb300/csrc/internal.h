@@ -1,6 +1,7 @@
 // Internal interfaces between the host library and the kernel translation units.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -21,6 +22,8 @@ struct PairArgs {
     float tau_ke;              // (1/eps_in - 1/eps_out) k_e
     float ke_out, kappa;       // k_e / eps_out and the salt's inverse Debye length (EF_SALT)
     float kc;                  // k_e / eps_in
+    float en_a, en_b, en_g;    // distant energy blocks (EnergyWide): set_energy_factors
+    float salt_l2;             // log2(eps_in / eps_out)
     float rep_k, rep_sigma;    // soft repulsion (rep_k == 0: off)
     float rgbmax;              // Born-radius cutoff (EF_CUT kernels of the Born and chain passes)
     float cut2;                // pair cutoff squared (EF_CUT kernels of the energy pass)
@@ -36,12 +39,20 @@ struct PairArgs {
     int* err;                  // device error word (non-finite input, nullable)
 };
 
-// One warp task: replica, super-row K (atoms 64K .. 64K+63), first tile J
-// (atoms 32J .. 32J+31, J >= 2K) and number of tiles; the walk continues
-// along the super-row, then into the next super-rows and replicas.
+// Replicas of up to this many 32-atom tiles (6400 atoms) run 64 x 32 blocks
+// only (walk_task in pairs_impl.cuh).  3 x 4999 atoms in salt water: 187 us a
+// force call with 64 x 32 blocks, 211 with 128 x 32; 16 x 4096 Born radii 148
+// against 183; 25,000-atom replicas the other way round (38.5 ms an MD step of
+// 48 with 128 x 32 blocks, 51 with the 64 x 32 ones before them).
+constexpr int SMALL_TILES = 200;
+
+// One warp task: replica, row pair and rows (4 P + 1, 2 or 3: atoms
+// 128P .. 128P+63, the 64 after them, or both), first tile J (atoms
+// 32J .. 32J+31, J >= 4P) and number of tiles of that row pair.
 struct TaskList {
     int4* d_tasks = nullptr;
     int n_tasks = 0;
+    bool small = false;        // every replica has at most SMALL_TILES tiles
     // register cap of each pass's kernel (Born, energy, chain), as 256-thread
     // blocks per SM: 1 (compiler's choice), 3 (80 registers) or 4 (64)
     int cap[3] = {1, 1, 1};
@@ -61,8 +72,8 @@ cudaError_t launch_pairs(int pass, int flags, const PairArgs& a, const TaskList&
 // Cutoff passes (pairs_cut.cu).  launch_block_list clears the LIST_CTRS
 // counters and builds the block neighbour lists from the tile boxes: list_b
 // (Born-radius cutoff, when want_b) and list_e (pair cutoff, when want_e),
-// each with room for every block of the batch; win_off [M+1] holds the first
-// list-building warp of each replica (ceil(nb/2) * ceil(nb/32) warps per
+// each with room for both rows of every column of the batch; win_off [M+1] holds the first
+// list-building warp of each replica (ceil(nb/4) * ceil(nb/32) warps per
 // replica of nb tiles).  launch_pairs_list runs pass `pass` with EF_CUT over
 // a device-built task list whose length is ctr[0] (Born, chain) or ctr[1]
 // (energy), taking tasks from the queue head ctr[2 + pass].
@@ -72,6 +83,17 @@ cudaError_t launch_block_list(const PairArgs& a, const int* win_off, int M, int 
 cudaError_t launch_pairs_list(int pass, int flags, const PairArgs& a, const int4* list, int* ctr, int cap,
                               int warps_per_block, cudaStream_t s);
 
+// Uniform factors of the distant energy blocks: with W = k_c q_i q_j / f^3
+// (times tF / k_c with salt, tau k_e / k_c folded into them without) the pair
+// adds W (en_a exp(-D) + en_b) to -(de/dr)/r and en_g W exp(-D) (1 + D) R_i R_j
+// to R de/dR.
+inline void set_energy_factors(PairArgs& a, const gb_params& p) {
+    const double tau = p.kappa != 0.0f ? 0.5 : 0.5 * (1.0 - (double)p.eps_in / (double)p.eps_out);
+    a.en_a = (float)(0.5 * tau);
+    a.en_b = (float)(-2.0 * tau);
+    a.en_g = (float)tau;
+    a.salt_l2 = (float)std::log2((double)p.eps_in / (double)p.eps_out);
+}
 // Cutoff fields of the pair arguments, and the EF_CUT flag of each pass.
 inline void set_cutoffs(PairArgs& a, const gb_params& p) {
     a.rgbmax = p.rgbmax;
@@ -89,8 +111,8 @@ inline bool params_ok(const gb_params& p) {
            p.rgbmax < 1.0e6f && p.cut >= 0.0f && p.cut < 1.0e6f;
 }
 
-// Work units (32-atom tiles against 64-atom super-rows) of an n-atom replica.
-int64_t pair_units(int64_t n);
+// Columns (32-atom tiles against 128-atom row pairs) of an n-atom replica.
+int64_t pair_columns(int64_t n);
 // Bounding boxes of all tiles (PairArgs::boxes, tile_off); no-op when boxes is null.
 cudaError_t launch_tile_boxes(const PairArgs& a, int M, int total_tiles, cudaStream_t s);
 

@@ -23,9 +23,14 @@
 namespace {
 
 constexpr int kMaxAtoms = GB_STATIC_MAX_ATOMS;
-constexpr int kTilesPerTask = 4;
-constexpr int kMaxTiles = (kMaxAtoms / 32) * (kMaxAtoms / 32 + 1) / 2;
-constexpr int kMaxTasks = (kMaxTiles + kTilesPerTask - 1) / kTilesPerTask;
+constexpr int kColsPerTask = 2;                  // runs of columns of a row pair, see pairs_impl.cuh
+// tasks of a molecule of nb tiles: row pair P has nb - 4P columns
+constexpr int static_tasks(int nb) {
+    int t = 0;
+    for (int c = nb; c > 0; c -= 4) t += (c + kColsPerTask - 1) / kColsPerTask;
+    return t;
+}
+constexpr int kMaxTasks = static_tasks(kMaxAtoms / 32);
 
 constexpr size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -74,11 +79,9 @@ int scratch_for_current_device(cudaStream_t s, unsigned char** out) {
     return GB_OK;
 }
 
-// Work list of one molecule: run w covers work units [w*tpt, (w+1)*tpt) of the
-// pair walk (super-rows K of 64 atoms against tiles J = 2K .. nb-1).  Also
-// writes atom_off = {0, n}.
-__global__ void k_static_tasks(int n, int nb, int tpt, int n_tasks, int64_t total, int4* tasks,
-                               int64_t* atom_off, int* ctr) {
+// Work list of one molecule: the columns of every row pair in runs of
+// kColsPerTask, one task each.  Also writes atom_off = {0, n}.
+__global__ void k_static_tasks(int n, int nb, int n_tasks, int4* tasks, int64_t* atom_off, int* ctr) {
     gbk::pdl_enter();
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w == 0) {
@@ -89,15 +92,14 @@ __global__ void k_static_tasks(int n, int nb, int tpt, int n_tasks, int64_t tota
         ctr[2] = ctr[3] = ctr[4] = 0;
     }
     if (w >= n_tasks) return;
-    int64_t p = (int64_t)w * tpt;
-    const int nk = (nb + 1) / 2;
-    int K = 0;
-    while (K < nk && p >= nb - 2 * K) {
-        p -= nb - 2 * K;
-        ++K;
+    int t = w, PR = 0;
+    for (int c = nb; c > 0; c -= 4, ++PR) {
+        const int k = (c + kColsPerTask - 1) / kColsPerTask;
+        if (t < k) break;
+        t -= k;
     }
-    const int64_t left = total - (int64_t)w * tpt;
-    tasks[w] = make_int4(0, K, 2 * K + (int)p, (int)(left < tpt ? left : tpt));
+    const int J = 4 * PR + t * kColsPerTask;
+    tasks[w] = make_int4(0, 4 * PR + 3, J, min(kColsPerTask, nb - J));
 }
 
 }  // namespace
@@ -116,8 +118,7 @@ extern "C" int gb_energy_forces_static(int32_t n_atoms, const gb_params* params,
     if (rc) return rc;
     const int n = n_atoms;
     const int nb = (n + 31) / 32;
-    const int64_t total = gbk::pair_units(n);
-    const int n_tasks = (int)((total + kTilesPerTask - 1) / kTilesPerTask);
+    const int n_tasks = static_tasks(nb);
 
     gbk::u64* I_acc = (gbk::u64*)(base + kOffI);
     gbk::u64* dR_acc = (gbk::u64*)(base + kOffDR);
@@ -134,8 +135,8 @@ extern "C" int gb_energy_forces_static(int32_t n_atoms, const gb_params* params,
 
     // the accumulators keep the last call's contents: start from zero
     if (cudaMemsetAsync(base, 0, kAccEnd, s) != cudaSuccess) return GB_ERR_CUDA;
-    if (gbk::launch_pdl(k_static_tasks, dim3((n_tasks + 255) / 256), dim3(256), 0, s, n, nb, kTilesPerTask, n_tasks,
-                        total, tasks, atom_off, ctr) != cudaSuccess)
+    if (gbk::launch_pdl(k_static_tasks, dim3((n_tasks + 255) / 256), dim3(256), 0, s, n, nb, n_tasks, tasks,
+                        atom_off, ctr) != cudaSuccess)
         return GB_ERR_CUDA;
 
     gbk::PairArgs pa{};
@@ -151,6 +152,7 @@ extern "C" int gb_energy_forces_static(int32_t n_atoms, const gb_params* params,
     pa.kappa = params->kappa;
     pa.rep_k = params->rep_k;
     pa.rep_sigma = params->rep_sigma;
+    gbk::set_energy_factors(pa, *params);
     gbk::set_cutoffs(pa, *params);
     pa.I_acc = I_acc;
     pa.dR_acc = dR_acc;

@@ -45,10 +45,10 @@ cudaError_t launch_pairs(int pass, int flags, const PairArgs& a, const TaskList&
     }
 }
 
-// Work units (tiles) of one replica of n atoms in the walk above.
-int64_t pair_units(int64_t n) {
-    const int64_t nb = (n + 31) / 32, nk = (nb + 1) / 2;
-    return nk * nb - nk * (nk - 1);
+// Columns of one replica of n atoms in the walk of pairs_impl.cuh.
+int64_t pair_columns(int64_t n) {
+    const int64_t nb = (n + 31) / 32, np = (nb + 3) / 4;
+    return np * nb - 2 * np * (np - 1);
 }
 
 }  // namespace gbk

@@ -2,11 +2,10 @@
 //
 // Every evaluation rebuilds the list from the tile bounding boxes of that
 // evaluation (k_tile_boxes, or k_md_step in the MD driver).  One warp covers
-// 32 consecutive blocks (K, J0 .. J0+31) of a super-row: lane l classifies
-// block (K, J0 + l) with cut_class, a ballot gives the warp the in-range bits,
-// and every run of consecutive in-range blocks (cut at 16 blocks) becomes one
-// task (replica, K, first J, length) of a compacted list, placed with one
-// atomic per warp.  Two lists: the Born-radius cutoff's (Born and chain
+// 32 consecutive columns J0 .. J0+31 of a row pair: lane l classifies the two
+// blocks of column J0 + l with cut_class, a ballot per row gives the warp the
+// bits of the blocks in range, and every run of them (cut at RUN) becomes one
+// task of a compacted list, placed with one atomic per row and warp.  Two lists: the Born-radius cutoff's (Born and chain
 // passes) and the pair cutoff's (energy pass).  The passes then take the
 // tasks from a queue (k_pairs_dyn): blocks out of range cost nothing, and
 // the warps' work evens out whatever the list's order.
@@ -20,16 +19,18 @@ namespace gbk {
 
 namespace {
 
+constexpr int RUN = 4;           // blocks per task at most (100,000 atoms, 12 A: 1.97 ms; 8: 2.05, 16: 2.27)
+
 __global__ void k_list_reset(int* ctr) {
     pdl_enter();
     if (threadIdx.x < LIST_CTRS) ctr[threadIdx.x] = 0;
 }
 
-// Appends the runs of set bits of m (lanes = blocks J0 ..) to a list.
-__device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int K, int J0, int4* list, int* counter) {
+// Appends the runs of set bits of m (lanes = columns J0 ..) to a list.
+__device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int row, int J0, int4* list, int* counter) {
     const bool on = (m >> lane) & 1u;
     const bool prev = lane > 0 && ((m >> (lane - 1)) & 1u);
-    const bool start = on && (!prev || (lane & 15) == 0);
+    const bool start = on && (!prev || (lane & (RUN - 1)) == 0);
     const unsigned sm = __ballot_sync(0xffffffffu, start);
     if (!sm) return;
     int base = 0;
@@ -38,13 +39,13 @@ __device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int K, in
     if (start) {
         const unsigned rest = ~(m >> lane);          // the run ends at the first zero
         int len = rest ? __ffs(rest) - 1 : 32 - lane;
-        len = min(len, 16 - (lane & 15));
-        list[base + __popc(sm & ((1u << lane) - 1u))] = make_int4(r, K, J0 + lane, len);
+        len = min(len, RUN - (lane & (RUN - 1)));
+        list[base + __popc(sm & ((1u << lane) - 1u))] = make_int4(r, row, J0 + lane, len);
     }
 }
 
-// win_off[r]: first warp of replica r; a replica has ceil(nb/2) super-rows of
-// ceil(nb/32) warps each (warps past the row's last block exit).
+// win_off[r]: first warp of replica r; a replica has ceil(nb/4) row pairs of
+// ceil(nb/32) warps each (warps past the row's last column exit).
 __global__ void k_block_list(PairArgs A, const int* __restrict__ win_off, int M, int total, int4* list_b,
                              int4* list_e, int* ctr, int want_b, int want_e) {
     pdl_enter();
@@ -62,21 +63,31 @@ __global__ void k_block_list(PairArgs A, const int* __restrict__ win_off, int M,
     const int nb = (n + 31) >> 5;
     const int wr = (nb + 31) >> 5;
     const int local = w - win_off[r];
-    const int K = local / wr;
-    const int J0 = 2 * K + 32 * (local % wr);
+    const int PR = local / wr;
+    const int J0 = 4 * PR + 32 * (local % wr);
     if (J0 >= nb) return;
     const int t0 = A.tile_off[r];
-    float4 ih;
-    const float4 il = row_box_lo(A, t0, K, nb, &ih);
     const int J = J0 + lane;
-    bool in_b = false, in_e = false, st;
+    bool in_b[2] = {false, false}, in_e[2] = {false, false};
     if (J < nb) {
-        const BoxPair b = box_pair(il, ih, __ldcg(&A.boxes[2 * (t0 + J)]), __ldcg(&A.boxes[2 * (t0 + J) + 1]));
-        if (want_b) cut_class(A, true, b, in_b, st);
-        if (want_e) cut_class(A, false, b, in_e, st);
+        const float4 jl = __ldcg(&A.boxes[2 * (t0 + J)]), jh = __ldcg(&A.boxes[2 * (t0 + J) + 1]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int K = 2 * PR + h;
+            if (J < 2 * K) continue;
+            float4 ih;
+            const float4 il = row_box_lo(A, t0, K, nb, &ih);
+            const BoxPair b = box_pair(il, ih, jl, jh);
+            bool st;
+            if (want_b) cut_class(A, true, b, in_b[h], st);
+            if (want_e) cut_class(A, false, b, in_e[h], st);
+        }
     }
-    if (want_b) emit_runs(__ballot_sync(0xffffffffu, in_b), lane, r, K, J0, list_b, &ctr[0]);
-    if (want_e) emit_runs(__ballot_sync(0xffffffffu, in_e), lane, r, K, J0, list_e, &ctr[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (want_b) emit_runs(__ballot_sync(0xffffffffu, in_b[h]), lane, r, 4 * PR + 1 + h, J0, list_b, &ctr[0]);
+        if (want_e) emit_runs(__ballot_sync(0xffffffffu, in_e[h]), lane, r, 4 * PR + 1 + h, J0, list_e, &ctr[1]);
+    }
 }
 
 constexpr int MAX_DEVICES = 64;
@@ -96,7 +107,7 @@ int resident_blocks(int wpb) {
     int& c = cache[current_device()][wpb];
     if (!c) {
         int per_sm = 0;
-        const size_t smem = (size_t)wpb * P::NQ * 64 * sizeof(long long);
+        const size_t smem = (size_t)wpb * WARP_SMEM<P>;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pairs_dyn<P, FLAGS, MINB>, 32 * wpb, smem) !=
                 cudaSuccess || per_sm < 1)
             per_sm = 1;
@@ -118,7 +129,8 @@ int sm_count() {
 
 template <class P, int FLAGS, int MINB>
 cudaError_t dyn_pass_cap(const PairArgs& a, const int4* list, int* ctr, int ci, int hi, int wpb, cudaStream_t s) {
-    const size_t smem = (size_t)wpb * P::NQ * 64 * sizeof(long long);
+    wpb = fit_warps<P>(wpb);
+    const size_t smem = (size_t)wpb * WARP_SMEM<P>;
     const int blocks = sm_count() * resident_blocks<P, FLAGS, MINB>(wpb);
     return launch_pdl(k_pairs_dyn<P, FLAGS, MINB>, dim3(blocks), dim3(32 * wpb), smem, s, a, list, ctr, ci, hi);
 }
@@ -127,7 +139,7 @@ template <class P, int FLAGS>
 cudaError_t dyn_pass(const PairArgs& a, const int4* list, int* ctr, int ci, int hi, int cap, int wpb,
                      cudaStream_t s) {
     if (cap >= 3) return dyn_pass_cap<P, FLAGS, 3>(a, list, ctr, ci, hi, wpb, s);
-    return dyn_pass_cap<P, FLAGS, 1>(a, list, ctr, ci, hi, wpb, s);
+    return dyn_pass_cap<P, FLAGS, 2>(a, list, ctr, ci, hi, wpb, s);
 }
 
 template <int F>

@@ -1,23 +1,24 @@
 // O(N^2) pair passes of the GB hot path on sm_103a.
 //
-// Every replica's atoms are cut into 32-atom tiles.  A warp owns a contiguous
-// run of the upper triangle's work, walked as 64-atom super-rows: lane l holds
-// the two atoms 64K + l and 64K + 32 + l ("i", one FP32x2 register pair per
-// quantity) for the whole row, while the 32 atoms of tile J ("j") rotate one
-// lane per step with warp shuffles, carrying their FP32 partial sums.  Each
-// step therefore evaluates two pairs per lane with packed FP32x2 arithmetic
-// (FFMA2 / FMUL2 / FADD2: one issue slot for two lanes' worth of FP32 work)
-// and one set of shuffles, and every unordered pair is evaluated exactly once
-// (Newton's third law).  The first two tiles of a super-row touch the
-// diagonal and are masked.  After each tile the j partials are folded into
-// int64 fixed point with one global atomic per atom and component; the i
-// partials go to int64 registers, flushed when the row ends.  FP32 partials
-// never span more than one 64 x 32 block and integer sums are associative,
-// so results are the same for every run, task split and launch order.
+// Every replica's atoms are cut into 32-atom tiles.  A warp owns runs of
+// blocks of the upper triangle: 64 or 128 atoms ("i", two or four a lane, one
+// FP32x2 register pair per two of them) against the 32 atoms of tile J ("j"),
+// which a lane meets one after the other while their FP32 partial sums rotate
+// one lane per step with warp shuffles.  Each step evaluates two or four
+// pairs per lane with packed FP32x2 arithmetic, and every unordered pair is
+// evaluated exactly once (Newton's third law).  The tiles on the diagonal are
+// masked.  After each tile the j partials are folded into int64 fixed point
+// with one global atomic per atom and component; the i partials go to int64
+// sums in shared memory, flushed when the task ends.  FP32 partials never span
+// more than one block and integer sums are associative, so results are the
+// same for every run, task split and launch order.
 //
 // Pass 1 (Born integrals), pass 2 (GB + Coulomb energy, direct forces, dE/dR,
 // optional dE/dq and soft repulsion) and pass 3 (Born-radius chain rule)
-// share the walker below; the arithmetic of each pass is in its policy.
+// share the walk (walk_task).  The general pair code of each pass (Born,
+// Energy, Chain) serves blocks that straddle a cutoff and evaluations that
+// want energies or dE/dq; every other block runs one of the forms under
+// "blocks by distance".
 #pragma once
 
 #include "common.cuh"
@@ -28,9 +29,7 @@ namespace gbk {
 
 // Disjoint spheres (r >= a + s) with x = s/r <= 0.6: H = 1/2 s^3 r^-4 g(x^2) and
 // -(dH/dr)/r = 1/2 s^3 r^-6 h(x^2), with g, h the fitted polynomials: no
-// cancellation and no MUFU.  Every lane evaluates the polynomial; the closed
-// form runs only when some lane of the warp holds an overlapping pair (a warp
-// vote), so the common path carries no divergent branch.
+// cancellation and no MUFU.
 __device__ __forceinline__ bool far_ok(float r, float lim, float y) { return (r >= lim) && (y <= GB_POLY_YMAX); }
 
 // True (warp-uniform) when every pair of this warp step has y <= GB_POLY_YFAR,
@@ -73,6 +72,11 @@ constexpr float LN2 = 0.69314718055994531f;
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr float FAR_R2 = 1.0e30f;                  // r^2 given to masked-off lanes
 
+__device__ __forceinline__ void set2(f2& v, int half, float x) {
+    if (half) v.y = x;
+    else v.x = x;
+}
+__device__ __forceinline__ float get2(f2 v, int half) { return half ? v.y : v.x; }
 __device__ __forceinline__ f2 neg2(f2 v) { return make_float2(-v.x, -v.y); }
 // Compensated summation (Kahan): sum + c carries the running total, with c
 // the negated rounding error of the additions so far.
@@ -93,6 +97,8 @@ __device__ __forceinline__ f2 rcp2(f2 x) {
     const f2 y = make_float2(rcp_ftz(x.x), rcp_ftz(x.y));
     return fma2(y, fma2(neg2(x), y, F2(1.0f)), y);
 }
+// the bare MUFU reciprocal (1 ulp), for the distant forms in 1/r^2
+__device__ __forceinline__ f2 rcp2_approx(f2 x) { return make_float2(rcp_ftz(x.x), rcp_ftz(x.y)); }
 __device__ __forceinline__ f2 logv(f2 x) { return make_float2(logf(x.x), logf(x.y)); }
 
 // --- HCT descreening integral H(r; a, s), closed form -----------------------------
@@ -354,15 +360,13 @@ __device__ __forceinline__ void load_xas(const PairArgs& A, int64_t base, int n,
 // --- pass 1: Born integrals I_i = sum_j H(r_ij; a_i, s_j) -----------------------
 struct Born {
     static constexpr int NQ = 1;      // int64 i-side accumulators per atom (shared memory)
-    static constexpr int UNROLL = 2;  // rotation steps unrolled (measured best per pass) ...
-    static constexpr int UNROLL_FAR = 4;   // ... and in far blocks
+    static constexpr int NJ = 1;      // j-side ones that close pairs add to
     static constexpr bool RADIUS_CUT = true;   // EF_CUT: the cutoff is rgbmax
+    static constexpr bool CHAIN = false;
     struct IState {
         f2 nx, ny, nz, a, s, s2, hs3;   // nx = -x
     };
-    // s2 = s^2 and hs3 = s^3 / 2 travel with the j atom through far blocks
-    // (one shuffle more, three multiplies fewer per step)
-    struct JState { float x, y, z, a, s, acc, s2, hs3; };
+    struct JState { float x, y, z, a, s, acc; };
     struct Part {
         f2 I;
         __device__ __forceinline__ void zero() { I = F2(0.0f); }
@@ -379,22 +383,18 @@ struct Born {
     static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, JState& st) {
         load_xas(A, base, n, j, st.x, st.y, st.z, st.a, st.s);
         st.acc = 0.0f;
-        st.s2 = st.s * st.s;
-        st.hs3 = 0.5f * st.s2 * st.s;
     }
     template <int FLAGS, int MODE, bool FAR>
     static __device__ __forceinline__ void pair(const PairArgs& A, const IState& i, JState& j, Part& p, Mask m,
                                                 const BlockInfo& bi, int, int, int) {
         const f2 dx = add2(F2(j.x), i.nx), dy = add2(F2(j.y), i.ny), dz = add2(F2(j.z), i.nz);
         const f2 r2 = safe_r2<MODE>(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), m);
-        // near blocks hold the few large terms that dominate an atom's
-        // integral (and the closed form, which cancels its terms about
-        // tenfold): there 1/r gets a Newton step, since the MUFU estimate's
-        // error enters r^-4 four times; far blocks sum many small terms
-        const f2 rinv = FAR ? rsqrt2(r2) : rsqrt2_nr(r2);
+        // the MUFU estimate's error enters r^-4 four times, and the closed
+        // form cancels its terms about tenfold: 1/r gets a Newton step
+        const f2 rinv = rsqrt2_nr(r2);
         const f2 rinv2 = mul2(rinv, rinv), rinv4 = mul2(rinv2, rinv2);
-        const float sj2 = FAR ? j.s2 : j.s * j.s;
-        const float hs3j = FAR ? j.hs3 : 0.5f * sj2 * j.s;
+        const float sj2 = j.s * j.s;
+        const float hs3j = 0.5f * sj2 * j.s;
         const f2 y_ij = mul2(F2(sj2), rinv2), y_ji = mul2(i.s2, rinv2);
         // EF_STRADDLE: lanes whose sphere lies wholly past rgbmax give 0; a step
         // with some sphere across it takes the restricted form for every lane
@@ -413,12 +413,6 @@ struct Born {
                 j.acc += h_ji.x + h_ji.y;
                 return;
             }
-        }
-        if (FAR) {  // whole block proven disjoint and far: no votes, short polynomial
-            p.I = fma2(F2(hs3j), mul2(rinv4, gb_poly_gf2(y_ij)), p.I);
-            const f2 h = mul2(i.hs3, mul2(rinv4, gb_poly_gf2(y_ji)));
-            j.acc += h.x + h.y;
-            return;
         }
         // the block bound t_near decides most steps with one compare per lane;
         // the exact per-direction tests run only on steps where some pair is
@@ -461,14 +455,9 @@ struct Born {
         j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
         j.a = shfl(j.a, src); j.s = shfl(j.s, src);
     }
-    // far blocks never read a: it is left behind (the block reloads it)
-    static __device__ __forceinline__ void rotate_far(JState& j, int src) {
-        j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
-        j.s2 = shfl(j.s2, src); j.hs3 = shfl(j.hs3, src);
-    }
     static __device__ __forceinline__ void rotate_acc(JState& j, int src) { j.acc = shfl(j.acc, src); }
     static __device__ __forceinline__ void take_data(JState& j, const JState& d) {
-        j.x = d.x; j.y = d.y; j.z = d.z; j.a = d.a; j.s = d.s; j.s2 = d.s2; j.hs3 = d.hs3;
+        j.x = d.x; j.y = d.y; j.z = d.z; j.a = d.a; j.s = d.s;
     }
     static __device__ __forceinline__ void fold_i(IState&, long long* sa, int lane, const Part& p) {
         sa[lane] += fix_i(p.I.x);
@@ -483,8 +472,9 @@ struct Born {
         if (!isfinite(st.acc) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
         if (j < n) red_add(&A.I_acc[base + j], fix_i(st.acc));
     }
-    static __device__ __forceinline__ void flush_i(const PairArgs& A, int, int64_t base, int n, int i0, int lane,
-                                                   const IState&, long long* sa) {
+    static __device__ __forceinline__ void flush_sums(const PairArgs&, int, int, const IState&) {}
+    static __device__ __forceinline__ void flush_i(const PairArgs& A, int64_t base, int n, int i0, int lane,
+                                                   long long* sa) {
         if (i0 + lane < n) red_add(&A.I_acc[base + i0 + lane], sa[lane]);
         if (i0 + 32 + lane < n) red_add(&A.I_acc[base + i0 + 32 + lane], sa[32 + lane]);
     }
@@ -502,9 +492,9 @@ struct Born {
 // exp(-D) = 2^(r^2 (-h_i) h_j) is two multiplies and one ex2.
 struct Energy {
     static constexpr int NQ = 5;      // fx, fy, fz, R dE/dR, dE/dq (shared memory)
-    static constexpr int UNROLL = 2;
-    static constexpr int UNROLL_FAR = 2;
+    static constexpr int NJ = 3;
     static constexpr bool RADIUS_CUT = false;  // EF_CUT: the cutoff is `cut`
+    static constexpr bool CHAIN = false;
     struct IState {
         f2 nx, ny, nz, q, R, nh;
         f2 qa, qk;                    // q tau k_e / 2 and q k_c (unscreened pair factors)
@@ -632,7 +622,6 @@ struct Energy {
         j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
         j.q = shfl(j.q, src); j.R = shfl(j.R, src); j.h = shfl(j.h, src);
     }
-    static __device__ __forceinline__ void rotate_far(JState& j, int src) { rotate_data(j, src); }
     template <int FLAGS>
     static __device__ __forceinline__ void rotate_acc_f(JState& j, int src) {
         j.fx = shfl(j.fx, src); j.fy = shfl(j.fy, src); j.fz = shfl(j.fz, src);
@@ -670,8 +659,8 @@ struct Energy {
         }
     }
     template <int FLAGS>
-    static __device__ __forceinline__ void flush_i_f(const PairArgs& A, int r, int64_t base, int n, int i0, int lane,
-                                                     const IState& st, long long* sa) {
+    static __device__ __forceinline__ void flush_i_f(const PairArgs& A, int64_t base, int n, int i0, int lane,
+                                                     long long* sa) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = i0 + 32 * h + lane;
@@ -685,6 +674,9 @@ struct Energy {
                 if (FLAGS & EF_PHI) red_add(&A.phi_acc[g], sa[256 + o]);
             }
         }
+    }
+    template <int FLAGS>
+    static __device__ __forceinline__ void flush_sums_f(const PairArgs& A, int r, int lane, const IState& st) {
         if (FLAGS & EF_ENERGY) {
             const long long egb = warp_sum_ll(st.egb), ec = warp_sum_ll(st.ec);
             const long long er = (FLAGS & EF_REP) ? warp_sum_ll(st.er) : 0;
@@ -703,14 +695,13 @@ struct Energy {
 //   -(dE/dr)/r = c_i * (-(dH(r; a_i, s_j)/dr)/r) + c_j * (-(dH(r; a_j, s_i)/dr)/r).
 struct Chain {
     static constexpr int NQ = 3;      // fx, fy, fz (shared memory)
-    static constexpr int UNROLL = 2;
-    static constexpr int UNROLL_FAR = 4;
+    static constexpr int NJ = 3;
     static constexpr bool RADIUS_CUT = true;   // EF_CUT: the cutoff is rgbmax
+    static constexpr bool CHAIN = true;
     struct IState {
         f2 nx, ny, nz, a, s, s2, hs3, c;
     };
-    // s2 = s^2 and hs3 = s^3 / 2 travel with the j atom through far blocks
-    struct JState { float x, y, z, a, s, c, fx, fy, fz, s2, hs3; };
+    struct JState { float x, y, z, a, s, c, fx, fy, fz; };
     struct Part {
         f2 sx, sy, sz;
         __device__ __forceinline__ void zero() { sx = sy = sz = F2(0.0f); }
@@ -732,8 +723,6 @@ struct Chain {
     static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, JState& st) {
         load_one(A, base, n, j, st.x, st.y, st.z, st.a, st.s, st.c);
         st.fx = st.fy = st.fz = 0.0f;
-        st.s2 = st.s * st.s;
-        st.hs3 = 0.5f * st.s2 * st.s;
     }
     template <int FLAGS, int MODE, bool FAR>
     static __device__ __forceinline__ void pair(const PairArgs& A, const IState& i, JState& j, Part& p, Mask m,
@@ -742,8 +731,8 @@ struct Chain {
         const f2 r2 = safe_r2<MODE>(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), m);
         const f2 rinv = rsqrt2(r2);
         const f2 rinv2 = mul2(rinv, rinv);
-        const float sj2 = FAR ? j.s2 : j.s * j.s;
-        const float hs3j = FAR ? j.hs3 : 0.5f * sj2 * j.s;
+        const float sj2 = j.s * j.s;
+        const float hs3j = 0.5f * sj2 * j.s;
         const f2 y_ij = mul2(F2(sj2), rinv2), y_ji = mul2(i.s2, rinv2);
         // EF_STRADDLE: as in Born; a lane with one direction wholly past rgbmax
         // has the other across it or past it too
@@ -764,16 +753,6 @@ struct Chain {
                 j.fz = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, j.fz));
                 return;
             }
-        }
-        if (FAR) {  // whole block proven disjoint and far: no votes, short polynomial
-            const f2 t = fma2(mul2(i.c, F2(hs3j)), gb_poly_hf2(y_ij),
-                              mul2(mul2(F2(j.c), i.hs3), gb_poly_hf2(y_ji)));
-            const f2 fr = mul2(t, mul2(rinv2, mul2(rinv2, rinv2)));
-            p.sx = fma2(fr, dx, p.sx); p.sy = fma2(fr, dy, p.sy); p.sz = fma2(fr, dz, p.sz);
-            j.fx = fmaf(fr.y, dx.y, fmaf(fr.x, dx.x, j.fx));
-            j.fy = fmaf(fr.y, dy.y, fmaf(fr.x, dy.x, j.fy));
-            j.fz = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, j.fz));
-            return;
         }
         // c_i s_j^3/2 h(y_ij) + c_j s_i^3/2 h(y_ji), times r^-6
         const float r2min = fminf(r2.x, r2.y);
@@ -817,15 +796,11 @@ struct Chain {
         j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
         j.a = shfl(j.a, src); j.s = shfl(j.s, src); j.c = shfl(j.c, src);
     }
-    static __device__ __forceinline__ void rotate_far(JState& j, int src) {
-        j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
-        j.s2 = shfl(j.s2, src); j.hs3 = shfl(j.hs3, src); j.c = shfl(j.c, src);
-    }
     static __device__ __forceinline__ void rotate_acc(JState& j, int src) {
         j.fx = shfl(j.fx, src); j.fy = shfl(j.fy, src); j.fz = shfl(j.fz, src);
     }
     static __device__ __forceinline__ void take_data(JState& j, const JState& d) {
-        j.x = d.x; j.y = d.y; j.z = d.z; j.a = d.a; j.s = d.s; j.c = d.c; j.s2 = d.s2; j.hs3 = d.hs3;
+        j.x = d.x; j.y = d.y; j.z = d.z; j.a = d.a; j.s = d.s; j.c = d.c;
     }
     static __device__ __forceinline__ void fold_i(IState&, long long* sa, int lane, const Part& p) {
         sa[lane] -= fix(p.sx.x); sa[32 + lane] -= fix(p.sx.y);
@@ -840,8 +815,9 @@ struct Chain {
             red_add(&A.F_acc[2 * A.N + g], fix(st.fz));
         }
     }
-    static __device__ __forceinline__ void flush_i(const PairArgs& A, int, int64_t base, int n, int i0, int lane,
-                                                   const IState&, long long* sa) {
+    static __device__ __forceinline__ void flush_sums(const PairArgs&, int, int, const IState&) {}
+    static __device__ __forceinline__ void flush_i(const PairArgs& A, int64_t base, int n, int i0, int lane,
+                                                   long long* sa) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = i0 + 32 * h + lane;
@@ -866,9 +842,12 @@ struct EnergyF : Energy {
     static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t b, int n, int j, const JState& s) {
         flush_j_f<FLAGS>(A, b, n, j, s);
     }
-    static __device__ __forceinline__ void flush_i(const PairArgs& A, int r, int64_t b, int n, int i0, int lane,
-                                                   const IState& s, long long* sa) {
-        flush_i_f<FLAGS>(A, r, b, n, i0, lane, s, sa);
+    static __device__ __forceinline__ void flush_i(const PairArgs& A, int64_t b, int n, int i0, int lane,
+                                                   long long* sa) {
+        flush_i_f<FLAGS>(A, b, n, i0, lane, sa);
+    }
+    static __device__ __forceinline__ void flush_sums(const PairArgs& A, int r, int lane, const IState& s) {
+        flush_sums_f<FLAGS>(A, r, lane, s);
     }
 };
 
@@ -884,14 +863,13 @@ __device__ __forceinline__ void run_tile(const PairArgs& A, const typename P::IS
     constexpr int K0 = (MODE == M_DX) ? 1 : 0, K1 = (MODE == M_DX) ? 17 : 32;
     // straddling blocks carry the long restricted-integral code: not unrolled,
     // so that it fits the instruction cache
-    constexpr int U = (FLAGS & EF_STRADDLE) ? 1 : (FAR ? P::UNROLL_FAR : P::UNROLL);
+    constexpr int U = (FLAGS & EF_STRADDLE) ? 1 : 2;
 #pragma unroll U
     for (int k = K0; k < K1; ++k) {
         // the next step's j data are fetched before this step's arithmetic, so
         // that only the short accumulator chain is serial between steps
         typename P::JState nx = js;
-        if (FAR) P::rotate_far(nx, next);
-        else P::rotate_data(nx, next);
+        P::rotate_data(nx, next);
         const Mask m = step_mask<MODE>(k, lane);
         bool busy = true;
         if (FLAGS & EF_STRADDLE) {   // every pair of this step wholly past the cutoff's reach
@@ -1002,71 +980,870 @@ __device__ __forceinline__ BlockInfo block_info(const PairArgs& A, int r, int K,
     return bi;
 }
 
-// Work of replica r is walked as super-rows K = 0 .. ceil(nb/2) - 1 (nb tiles
-// of 32 atoms), each over tiles J = 2K .. nb-1; a task is (replica, K, J,
-// number of tiles) and may continue into the next super-rows and replicas.
-// One warp task walks (replica, K, J, count); sa is the warp's shared-memory
-// slot of P::NQ x 64 int64 i-side accumulators (each lane owns its two atoms'
-// entries).  Loads of data that kernels rewrite (coordinates, radii, chain
-// factors, boxes) go through L2 (ld.global.cg): a persistent launch reads
-// them again after other SMs changed them, and L1 is not coherent.
-template <class P, int FLAGS>
-__device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, long long* sa, int lane) {
+// --- blocks by distance ---------------------------------------------------------------
+// Every 64 x 32 block is classified from the tile boxes (row_tier).  For the
+// Born and chain passes
+//   near (0):     some pair may overlap or have (s/r)^2 > GB_POLY_YFAR;
+//                 polynomials in y = (s/r)^2 up to GB_POLY_YNEAR;
+//   far (1):      none has: polynomials in y of degree 4 and 5;
+//   distant (2, 3): polynomials of degree 3 or 2 in u = 1/r^2 with the powers
+//                 of s folded into per-atom coefficients,
+//                   H(r; a, s) = u^2 (A_0 + A_1 u + ...),  A_k = 1/2 s^3 g_k s^2k
+//                   -(dH/dr)/r = u^3 (B_0 + B_1 u + ...),  B_k = 1/2 s^3 h_k s^2k
+//                 (GB_Y_*: the largest (s/r)^2 for which such a fit is as good
+//                 as the FP32 form that nearer blocks use).
+// The integrals contain even powers of r only, so 1/r^2 is one MUFU
+// reciprocal and no square root is taken.  The energy pass has one form; its
+// near blocks are those inside the soft repulsion's range.
+//
+// Where both rows of a row pair are far from a tile the block is evaluated
+// 128 x 32: lane l holds the four atoms 128 P + 32 q + l (NW = 2 FP32x2
+// pairs), so that one load of the j atom and one rotation of its partial sums
+// serve four pairs a lane.  A pair step costs issue slots for everything it
+// executes -- an FP32x2 instruction takes two, three when it reads three
+// different register pairs -- so shuffles and moves count in full: at two
+// atoms a lane with the j atoms rotated by shuffles they were a third of the
+// 72 / 110 / 104 slots of a Born / energy / chain step of 64 pairs, which now
+// takes 36 to 41 / 79 / 57 to 62.
+//
+// Near and diagonal blocks (64 x 32, NW = 1) run the far form for every pair,
+// without votes or branches; pairs closer than the block's bound t are left
+// out (r^2 set to FAR_R2) and noted in a bit mask.  After the tile those are
+// gathered and evaluated 32 at a time, exactly (close_pairs): two pairs of a
+// hundred, which otherwise made every second step of a near block run the
+// closed form for all its lanes.
+
+// r^2 of a step's pairs: masked-off pairs (diagonal blocks) read as far; with
+// NEAR, pairs below t set bit `bit` of the lane's masks and, with DROP, read
+// as far too.
+template <int MODE, bool NEAR, bool DROP>
+__device__ __forceinline__ f2 screen_r2(f2 r2, Mask m, float t, unsigned bit, unsigned& mx, unsigned& my) {
+    if (MODE == M_FULL && !NEAR) return r2;
+    const bool cx = NEAR && r2.x < t && m.x, cy = NEAR && r2.y < t && m.y;
+    if (NEAR) {
+        mx |= cx ? bit : 0u;
+        my |= cy ? bit : 0u;
+    }
+    return make_float2((DROP && cx) || !m.x ? FAR_R2 : r2.x, (DROP && cy) || !m.y ? FAR_R2 : r2.y);
+}
+
+// The staged tile of a warp: j atoms (twice, see stage()), what close pairs
+// need of both sides, their j sums and their queue.
+constexpr int CLOSE_CAP = 512;
+template <class W>
+struct Slot {
+    long long* sa;        // [2][NQ][64] i-side sums of both rows
+    float4* j4;           // [64] x, y, z and a fourth value of the j atoms
+    typename W::B* jb;    // [64] further values
+    float2* ja;           // [32] a, s of the j atoms
+    long long* jac;       // [NJ][32] j-side sums of close pairs
+    float4* i4;           // [64] x, y, z, c of the i atoms
+    float2* i2;           // [64] a, s of the i atoms
+    unsigned short* queue;
+    __device__ __forceinline__ explicit Slot(int slot) {
+        extern __shared__ __align__(16) unsigned char s_mem[];
+        unsigned char* p = s_mem + slot;
+        sa = (long long*)p;
+        j4 = (float4*)(p + 2 * W::NQ * 64 * 8);
+        jb = (typename W::B*)(j4 + 64);
+        ja = (float2*)(j4 + 96);
+        jac = (long long*)(ja + 32);
+        i4 = (float4*)(jac + 32 * W::NJ);
+        i2 = (float2*)(i4 + 64);
+        queue = (unsigned short*)(i2 + 64);
+    }
+};
+// Shared memory of a warp: i-side sums of two rows, then the larger of the
+// staged tile of 128 x 32 blocks (two float4 arrays of 64) and a Slot.
+template <class P>
+constexpr int WARP_SMEM = 2 * P::NQ * 64 * 8 + 1024 + 512 + 256 + P::NJ * 256 + 1024 + 512 + 2 * CLOSE_CAP;
+// Warps per block a pass can run within the 48 KB that need no opt-in.
+template <class P>
+inline int fit_warps(int wpb) { return wpb * WARP_SMEM<P> <= 49152 ? wpb : 49152 / WARP_SMEM<P>; }
+
+// Exact sum into a shared 64-bit word by two 32-bit atomics (there is no
+// native 64-bit one): the carry follows from the low word's old value.
+__device__ __forceinline__ void shared_add(long long* p, long long v) {
+    unsigned* w = (unsigned*)p;
+    const unsigned lo = (unsigned)v;
+    unsigned hi = (unsigned)((u64)v >> 32);
+    const unsigned old = atomicAdd(w, lo);
+    hi += (old + lo < lo) ? 1u : 0u;
+    if (hi) atomicAdd(w + 1, hi);
+}
+
+// The r^2 below which a pair of a near block is close: above it the spheres
+// are disjoint in both directions and (s/r)^2 <= GB_POLY_YNEAR.  Rounded up a
+// little, so that rounding in r^2 cannot admit a pair that is neither.
+__device__ __forceinline__ float close_bound(float amax, float smax) {
+    const float as = amax + smax;
+    return 1.0001f * fmaxf(as * as, smax * smax * (1.0f / GB_POLY_YNEAR));
+}
+// The same from the staged atoms, where there are no tile boxes.
+template <class W>
+__device__ __forceinline__ float staged_bound(const Slot<W>& S, int lane) {
+    const float2 a = S.i2[lane], b = S.i2[32 + lane], c = S.ja[lane];
+    float am = fmaxf(a.x, fmaxf(b.x, c.x)), sm = fmaxf(a.y, fmaxf(b.y, c.y));
 #pragma unroll
-    for (int q = 0; q < 2 * P::NQ; ++q) sa[32 * q + lane] = 0;
-    int r = t.x, K = t.y, J = t.z;
-    const int cnt = t.w;
-    int64_t base = A.atom_off[r];
-    int n = (int)(A.atom_off[r + 1] - base);
-    int nb = (n + 31) >> 5;
-    int nk = (nb + 1) >> 1;
+    for (int o = 16; o > 0; o >>= 1) {
+        am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
+        sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, o));
+    }
+    return close_bound(am, sm);
+}
+
+// --- Born integrals --------------------------------------------------------------------
+template <int NW>
+struct BornY {
+    static constexpr int ATOMS = 64 * NW, NQ = Born::NQ, NJ = Born::NJ, UNROLL = NW == 2 ? 2 : 4;
+    struct I { f2 nx[NW], ny[NW], nz[NW], s2[NW], hs3[NW]; };
+    typedef float B;                                   // staged j values: x, y, z, s^2 | s^3 / 2
+    struct J { float acc; };
+    struct Part { f2 s[NW]; };
+    static __device__ __forceinline__ void load(const PairArgs& A, int64_t base, int n, int i, float4& v, B& b, float2& as) {
+        load_xas(A, base, n, i, v.x, v.y, v.z, as.x, as.y);
+        v.w = as.y * as.y;
+        b = 0.5f * v.w * as.y;
+    }
+    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, I& st,
+                                                  float4* i4 = nullptr, float2* i2 = nullptr) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) {
+            float4 v;
+            float b;
+            float2 as;
+            load(A, base, n, i0 + 32 * q + lane, v, b, as);
+            set2(st.nx[q >> 1], q & 1, -v.x); set2(st.ny[q >> 1], q & 1, -v.y); set2(st.nz[q >> 1], q & 1, -v.z);
+            set2(st.s2[q >> 1], q & 1, v.w); set2(st.hs3[q >> 1], q & 1, b);
+            if (i4) {
+                i4[32 * q + lane] = v;
+                i2[32 * q + lane] = as;
+            }
+        }
+    }
+    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, float4& v, B& b) {
+        float2 as;
+        load(A, base, n, j, v, b, as);
+    }
+    static __device__ __forceinline__ void zero(J& j, Part& p) {
+        j.acc = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) p.s[q] = F2(0.0f);
+    }
+    template <int MODE = M_FULL, bool NEAR = false>
+    static __device__ __forceinline__ void step(const PairArgs&, const I& i, float4 v, B b, J& j, Part& p,
+                                                Mask m = Mask{true, true}, float t = 0.0f, unsigned bit = 0,
+                                                unsigned* mk = nullptr) {
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const f2 dx = add2(F2(v.x), i.nx[q]), dy = add2(F2(v.y), i.ny[q]), dz = add2(F2(v.z), i.nz[q]);
+            f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+            if (MODE != M_FULL || NEAR) r2 = screen_r2<MODE, NEAR, true>(r2, m, t, bit, mk[0], mk[1]);
+            const f2 u = rcp2_approx(r2);
+            const f2 u2 = mul2(u, u);
+            const f2 yj = mul2(F2(v.w), u), yi = mul2(i.s2[q], u);
+            p.s[q] = fma2(F2(b), mul2(u2, NW == 1 ? gb_poly_gn2(yj) : gb_poly_gf2(yj)), p.s[q]);
+            const f2 h = mul2(u2, NW == 1 ? gb_poly_gn2(yi) : gb_poly_gf2(yi));
+            j.acc = fmaf(i.hs3[q].y, h.y, fmaf(i.hs3[q].x, h.x, j.acc));
+        }
+    }
+    static __device__ __forceinline__ void rotate_acc(J& j, int src) { j.acc = shfl(j.acc, src); }
+    static __device__ __forceinline__ void fold_i(const PairArgs&, long long* sa, int lane, const Part& p) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) sa[32 * q + lane] += fix_i(get2(p.s[q >> 1], q & 1));
+    }
+    // Two atoms at the same position (r = 0; masked pairs read as far) give a
+    // NaN through r = r^2 / r; a NaN coordinate gives one in every sum it
+    // enters.  Both are recorded before the fixed-point conversion would
+    // hide them: here and where close pairs are evaluated.
+    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const J& st,
+                                                   const long long* jac = nullptr, int at = 0) {
+        if (!isfinite(st.acc) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
+        if (j < n) red_add(&A.I_acc[base + j], fix_i(st.acc) + (jac ? jac[at] : 0));
+    }
+    static __device__ __forceinline__ float bound(const PairArgs&, const Slot<BornY>& S, int lane) { return staged_bound(S, lane); }
+    // One close pair a lane, both directions as the halves of a pair.
+    static __device__ __forceinline__ void close(const PairArgs& A, const Slot<BornY>& S, long long* sa, int i, int j,
+                                                 bool valid, int, int) {
+        const float4 xi = S.i4[i], xj = S.j4[j];
+        const float2 ai = S.i2[i], aj = S.ja[j];
+        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+        const f2 r2 = F2(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        const f2 rinv = rsqrt2_nr(r2), r = mul2(r2, rinv), rinv2 = mul2(rinv, rinv);
+        const f2 a = make_float2(ai.x, aj.x), s = make_float2(aj.y, ai.y), s2 = mul2(s, s);
+        const f2 y = mul2(s2, rinv2);
+        f2 h = mul2(mul2(mul2(F2(0.5f), s2), s), mul2(mul2(rinv2, rinv2), gb_poly_g2(y)));
+        const bool c0 = !far_ok(r.x, a.x + s.x, y.x), c1 = !far_ok(r.y, a.y + s.y, y.y);
+        if (__any_sync(0xffffffffu, c0 || c1)) {
+            const f2 hc = hct_closed2(r, rinv, a, s);
+            h = make_float2(c0 ? hc.x : h.x, c1 ? hc.y : h.y);
+        }
+        if (!valid) return;
+        if (!isfinite(h.x + h.y) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
+        shared_add(&sa[i], fix_i(h.x));
+        shared_add(&S.jac[j], fix_i(h.y));
+    }
+};
+
+template <int NW, int DEG>
+struct BornU {
+    static constexpr int ATOMS = 64 * NW, NQ = Born::NQ, UNROLL = 2;
+    struct I { f2 nx[NW], ny[NW], nz[NW], A[NW][DEG + 1]; };
+    typedef float4 B;                                  // staged j values: x, y, z, A_0 | A_1 ...
+    struct J { float acc; };
+    struct Part { f2 s[NW]; };
+    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, float4& v, B& b) {
+        constexpr float g3[] = GB_G3, g2[] = GB_G2;
+        float a, s, c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        load_xas(A, base, n, j, v.x, v.y, v.z, a, s);
+        float h = 0.5f * s * s * s;
+#pragma unroll
+        for (int k = 0; k <= DEG; ++k) {
+            c[k] = h * (DEG == 3 ? g3[k] : g2[k]);
+            h *= s * s;
+        }
+        v.w = c[0];
+        b = make_float4(c[1], c[2], c[3], 0.0f);
+    }
+    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, I& st) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) {
+            float4 v;
+            B b;
+            load_j(A, base, n, i0 + 32 * q + lane, v, b);
+            const float c[4] = {v.w, b.x, b.y, b.z};
+            set2(st.nx[q >> 1], q & 1, -v.x); set2(st.ny[q >> 1], q & 1, -v.y); set2(st.nz[q >> 1], q & 1, -v.z);
+#pragma unroll
+            for (int k = 0; k <= DEG; ++k) set2(st.A[q >> 1][k], q & 1, c[k]);
+        }
+    }
+    static __device__ __forceinline__ void zero(J& j, Part& p) {
+        j.acc = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) p.s[q] = F2(0.0f);
+    }
+    static __device__ __forceinline__ void step(const PairArgs&, const I& i, float4 v, B b, J& j, Part& p) {
+        const float c[4] = {v.w, b.x, b.y, b.z};
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const f2 dx = add2(F2(v.x), i.nx[q]), dy = add2(F2(v.y), i.ny[q]), dz = add2(F2(v.z), i.nz[q]);
+            const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+            const f2 u = rcp2_approx(r2);
+            const f2 u2 = mul2(u, u);
+            f2 pj = F2(c[DEG]), pi = i.A[q][DEG];
+#pragma unroll
+            for (int k = DEG - 1; k >= 0; --k) {
+                pj = fma2(u, pj, F2(c[k]));
+                pi = fma2(u, pi, i.A[q][k]);
+            }
+            p.s[q] = fma2(u2, pj, p.s[q]);
+            j.acc = fmaf(u2.y, pi.y, fmaf(u2.x, pi.x, j.acc));
+        }
+    }
+    static __device__ __forceinline__ void rotate_acc(J& j, int src) { j.acc = shfl(j.acc, src); }
+    static __device__ __forceinline__ void fold_i(const PairArgs&, long long* sa, int lane, const Part& p) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) sa[32 * q + lane] += fix_i(get2(p.s[q >> 1], q & 1));
+    }
+    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const J& st) {
+        if (!isfinite(st.acc) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
+        if (j < n) red_add(&A.I_acc[base + j], fix_i(st.acc));
+    }
+};
+
+// --- chain rule ------------------------------------------------------------------------
+// Force sums of a pass whose blocks add fr d to j and -fr d to i.
+template <int NW>
+struct ForceSums {
+    struct J { float fx, fy, fz; };
+    struct Part { f2 x[NW], y[NW], z[NW]; };
+    static __device__ __forceinline__ void zero(J& j, Part& p) {
+        j.fx = j.fy = j.fz = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) p.x[q] = p.y[q] = p.z[q] = F2(0.0f);
+    }
+    static __device__ __forceinline__ void add(f2 fr, f2 dx, f2 dy, f2 dz, int q, J& j, Part& p) {
+        p.x[q] = fma2(fr, dx, p.x[q]); p.y[q] = fma2(fr, dy, p.y[q]); p.z[q] = fma2(fr, dz, p.z[q]);
+        j.fx = fmaf(fr.y, dx.y, fmaf(fr.x, dx.x, j.fx));
+        j.fy = fmaf(fr.y, dy.y, fmaf(fr.x, dy.x, j.fy));
+        j.fz = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, j.fz));
+    }
+    static __device__ __forceinline__ void rotate_acc(J& j, int src) {
+        j.fx = shfl(j.fx, src); j.fy = shfl(j.fy, src); j.fz = shfl(j.fz, src);
+    }
+    template <int NQ>
+    static __device__ __forceinline__ void fold(long long* sa, int lane, const Part& p) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) {
+            long long* o = sa + (q >> 1) * 64 * NQ + 32 * (q & 1) + lane;
+            o[0] -= fix(get2(p.x[q >> 1], q & 1));
+            o[64] -= fix(get2(p.y[q >> 1], q & 1));
+            o[128] -= fix(get2(p.z[q >> 1], q & 1));
+        }
+    }
+    static __device__ __forceinline__ void flush(const PairArgs& A, int64_t g, const J& st, const long long* jac, int at) {
+        red_add(&A.F_acc[g], fix(st.fx) + (jac ? jac[at] : 0));
+        red_add(&A.F_acc[A.N + g], fix(st.fy) + (jac ? jac[32 + at] : 0));
+        red_add(&A.F_acc[2 * A.N + g], fix(st.fz) + (jac ? jac[64 + at] : 0));
+    }
+    // a close pair's force fr d, exactly
+    static __device__ __forceinline__ void add_close(long long* sa, long long* jac, int i, int j, float fr, float dx,
+                                                     float dy, float dz) {
+        const long long fx = fix(fr * dx), fy = fix(fr * dy), fz = fix(fr * dz);
+        shared_add(&sa[i], -fx); shared_add(&sa[64 + i], -fy); shared_add(&sa[128 + i], -fz);
+        shared_add(&jac[j], fx); shared_add(&jac[32 + j], fy); shared_add(&jac[64 + j], fz);
+    }
+};
+
+template <int NW>
+struct ChainY : ForceSums<NW> {
+    typedef ForceSums<NW> F;
+    static constexpr int ATOMS = 64 * NW, NQ = Chain::NQ, NJ = Chain::NJ, UNROLL = NW == 2 ? 1 : 4;
+    struct I { f2 nx[NW], ny[NW], nz[NW], s2[NW], hs3[NW], c[NW]; };
+    typedef float2 B;                                  // staged j values: x, y, z, s^2 | s^3 / 2, c
+    static __device__ __forceinline__ void load(const PairArgs& A, int64_t base, int n, int i, float4& v, B& b, float2& as) {
+        Chain::load_one(A, base, n, i, v.x, v.y, v.z, as.x, as.y, b.y);
+        v.w = as.y * as.y;
+        b.x = 0.5f * v.w * as.y;
+    }
+    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, I& st,
+                                                  float4* i4 = nullptr, float2* i2 = nullptr) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) {
+            float4 v;
+            B b;
+            float2 as;
+            load(A, base, n, i0 + 32 * q + lane, v, b, as);
+            set2(st.nx[q >> 1], q & 1, -v.x); set2(st.ny[q >> 1], q & 1, -v.y); set2(st.nz[q >> 1], q & 1, -v.z);
+            set2(st.s2[q >> 1], q & 1, v.w); set2(st.hs3[q >> 1], q & 1, b.x); set2(st.c[q >> 1], q & 1, b.y);
+            if (i4) {
+                i4[32 * q + lane] = make_float4(v.x, v.y, v.z, b.y);
+                i2[32 * q + lane] = as;
+            }
+        }
+    }
+    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, float4& v, B& b) {
+        float2 as;
+        load(A, base, n, j, v, b, as);
+    }
+    template <int MODE = M_FULL, bool NEAR = false>
+    static __device__ __forceinline__ void step(const PairArgs&, const I& i, float4 v, B b, typename F::J& j,
+                                                typename F::Part& p, Mask m = Mask{true, true}, float t = 0.0f,
+                                                unsigned bit = 0, unsigned* mk = nullptr) {
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const f2 dx = add2(F2(v.x), i.nx[q]), dy = add2(F2(v.y), i.ny[q]), dz = add2(F2(v.z), i.nz[q]);
+            f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+            if (MODE != M_FULL || NEAR) r2 = screen_r2<MODE, NEAR, true>(r2, m, t, bit, mk[0], mk[1]);
+            const f2 u = rcp2_approx(r2);
+            const f2 yj = mul2(F2(v.w), u), yi = mul2(i.s2[q], u);
+            const f2 t1 = fma2(mul2(i.c[q], F2(b.x)), NW == 1 ? gb_poly_hn2(yj) : gb_poly_hf2(yj),
+                               mul2(mul2(F2(b.y), i.hs3[q]), NW == 1 ? gb_poly_hn2(yi) : gb_poly_hf2(yi)));
+            F::add(mul2(t1, mul2(u, mul2(u, u))), dx, dy, dz, q, j, p);
+        }
+    }
+    static __device__ __forceinline__ void fold_i(const PairArgs&, long long* sa, int lane, const typename F::Part& p) {
+        F::template fold<NQ>(sa, lane, p);
+    }
+    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const typename F::J& st,
+                                                   const long long* jac = nullptr, int at = 0) {
+        if (j < n) F::flush(A, base + j, st, jac, at);
+    }
+    static __device__ __forceinline__ float bound(const PairArgs&, const Slot<ChainY>& S, int lane) { return staged_bound(S, lane); }
+    static __device__ __forceinline__ void close(const PairArgs& A, const Slot<ChainY>& S, long long* sa, int i, int j,
+                                                 bool valid, int, int) {
+        const float4 xi = S.i4[i], xj = S.j4[j];
+        const float2 ai = S.i2[i], aj = S.ja[j];
+        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+        const f2 r2 = F2(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        const f2 rinv = rsqrt2_nr(r2), r = mul2(r2, rinv), rinv2 = mul2(rinv, rinv);
+        const f2 a = make_float2(ai.x, aj.x), s = make_float2(aj.y, ai.y), s2 = mul2(s, s);
+        const f2 y = mul2(s2, rinv2);
+        f2 h = mul2(mul2(mul2(F2(0.5f), s2), s), mul2(mul2(rinv2, mul2(rinv2, rinv2)), gb_poly_h2(y)));
+        const bool c0 = !far_ok(r.x, a.x + s.x, y.x), c1 = !far_ok(r.y, a.y + s.y, y.y);
+        if (__any_sync(0xffffffffu, c0 || c1)) {
+            const f2 hc = hct_closed_fr2(r, rinv, a, s);
+            h = make_float2(c0 ? hc.x : h.x, c1 ? hc.y : h.y);
+        }
+        if (valid) F::add_close(sa, S.jac, i, j, fmaf(xi.w, h.x, S.jb[j].y * h.y), dx, dy, dz);
+    }
+};
+
+template <int NW, int DEG>
+struct ChainU : ForceSums<NW> {
+    typedef ForceSums<NW> F;
+    static constexpr int ATOMS = 64 * NW, NQ = Chain::NQ, UNROLL = NW == 2 ? 1 : 2;
+    struct I { f2 nx[NW], ny[NW], nz[NW], c[NW], Bk[NW][DEG + 1]; };
+    typedef float4 B;                                  // staged j values: x, y, z, c | B_k
+    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, float4& v, B& b) {
+        constexpr float h3[] = GB_H3, h2[] = GB_H2;
+        float a, s, c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        Chain::load_one(A, base, n, j, v.x, v.y, v.z, a, s, v.w);
+        float h = 0.5f * s * s * s;
+#pragma unroll
+        for (int k = 0; k <= DEG; ++k) {
+            c[k] = h * (DEG == 3 ? h3[k] : h2[k]);
+            h *= s * s;
+        }
+        b = make_float4(c[0], c[1], c[2], c[3]);
+    }
+    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, I& st) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) {
+            float4 v;
+            B b;
+            load_j(A, base, n, i0 + 32 * q + lane, v, b);
+            const float c[4] = {b.x, b.y, b.z, b.w};
+            set2(st.nx[q >> 1], q & 1, -v.x); set2(st.ny[q >> 1], q & 1, -v.y); set2(st.nz[q >> 1], q & 1, -v.z);
+            set2(st.c[q >> 1], q & 1, v.w);
+#pragma unroll
+            for (int k = 0; k <= DEG; ++k) set2(st.Bk[q >> 1][k], q & 1, c[k]);
+        }
+    }
+    static __device__ __forceinline__ void step(const PairArgs&, const I& i, float4 v, B b, typename F::J& j, typename F::Part& p) {
+        const float c[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const f2 dx = add2(F2(v.x), i.nx[q]), dy = add2(F2(v.y), i.ny[q]), dz = add2(F2(v.z), i.nz[q]);
+            const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+            const f2 u = rcp2_approx(r2);
+            f2 pj = F2(c[DEG]), pi = i.Bk[q][DEG];
+#pragma unroll
+            for (int k = DEG - 1; k >= 0; --k) {
+                pj = fma2(u, pj, F2(c[k]));
+                pi = fma2(u, pi, i.Bk[q][k]);
+            }
+            const f2 t = fma2(i.c[q], pj, mul2(F2(v.w), pi));
+            F::add(mul2(t, mul2(u, mul2(u, u))), dx, dy, dz, q, j, p);
+        }
+    }
+    static __device__ __forceinline__ void fold_i(const PairArgs&, long long* sa, int lane, const typename F::Part& p) {
+        F::template fold<NQ>(sa, lane, p);
+    }
+    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const typename F::J& st) {
+        if (j < n) F::flush(A, base + j, st, nullptr, 0);
+    }
+};
+
+// --- GB + Coulomb forces and R dE/dR (no energies, no dE/dq) ----------------------------
+// With Q = k_c q_i q_j, W = Q / f^3 (times the screened factor with salt) and
+// E = exp(-D),
+//   -(de/dr)/r = Q / r^3 + W (en_a E + en_b),   R de/dR = en_g W E (R_i R_j + r^2/4):
+// the solvent constants sit in two uniform factors of the bracket and in one
+// factor applied when a block's sums are folded.
+template <int NW, int FLAGS>
+struct EnergyW : ForceSums<NW> {
+    typedef ForceSums<NW> F;
+    static constexpr int ATOMS = 64 * NW, NQ = Energy::NQ, NJ = Energy::NJ, UNROLL = NW == 2 ? 1 : 4;
+    struct I { f2 nx[NW], ny[NW], nz[NW], Q[NW], R[NW], nh[NW]; };
+    typedef float2 B;                                  // staged j values: x, y, z, q | R, h
+    struct J : F::J { float dR; };
+    struct Part : F::Part { f2 dR[NW]; };
+    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, float4& v, B& b) {
+        Energy::load_one(A, base, n, j, v.x, v.y, v.z, v.w, b.x, b.y);
+    }
+    static __device__ __forceinline__ void load(const PairArgs& A, int64_t base, int n, int i, float4& v, B& b, float2& as) {
+        load_j(A, base, n, i, v, b);
+        as = F2(0.0f);
+    }
+    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, I& st,
+                                                  float4* i4 = nullptr, float2* = nullptr) {
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q) {
+            float4 v;
+            B b;
+            load_j(A, base, n, i0 + 32 * q + lane, v, b);
+            set2(st.nx[q >> 1], q & 1, -v.x); set2(st.ny[q >> 1], q & 1, -v.y); set2(st.nz[q >> 1], q & 1, -v.z);
+            set2(st.Q[q >> 1], q & 1, v.w * A.kc);
+            set2(st.R[q >> 1], q & 1, b.x);
+            set2(st.nh[q >> 1], q & 1, -b.y);
+            if (i4) i4[32 * q + lane] = v;
+        }
+    }
+    static __device__ __forceinline__ void zero(J& j, Part& p) {
+        F::zero(j, p);
+        j.dR = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) p.dR[q] = F2(0.0f);
+    }
+    template <int MODE = M_FULL, bool NEAR = false>
+    static __device__ __forceinline__ void step(const PairArgs& A, const I& i, float4 v, B b, J& j, Part& p,
+                                                Mask m = Mask{true, true}, float t = 0.0f, unsigned bit = 0,
+                                                unsigned* mk = nullptr) {
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const f2 dx = add2(F2(v.x), i.nx[q]), dy = add2(F2(v.y), i.ny[q]), dz = add2(F2(v.z), i.nz[q]);
+            f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+            // pairs inside the repulsion's range keep their GB and Coulomb terms here
+            if (MODE != M_FULL || NEAR) r2 = screen_r2<MODE, NEAR, false>(r2, m, t, bit, mk[0], mk[1]);
+            const f2 rinv = rsqrt2(r2);
+            const f2 e = ex22(mul2(r2, mul2(i.nh[q], F2(b.y))));          // exp(-D)
+            const f2 RR = mul2(i.R[q], F2(b.x));
+            const f2 fsq = fma2(RR, e, r2);
+            const f2 finv = rsqrt2(fsq);
+            const f2 Q = mul2(i.Q[q], F2(v.w));
+            f2 W = mul2(mul2(Q, finv), mul2(finv, finv));
+            if (FLAGS & EF_SALT) {
+                // tF / k_c = 1 - (1 + kappa f) k, k = (eps_in / eps_out) exp(-kappa f)
+                const f2 kf = mul2(F2(A.kappa), mul2(fsq, finv));
+                const f2 k = ex22(fma2(F2(-LOG2E), kf, F2(A.salt_l2)));
+                W = mul2(W, fma2(neg2(k), kf, add2(F2(1.0f), neg2(k))));
+            }
+            const f2 fr = fma2(W, fma2(F2(A.en_a), e, F2(A.en_b)), mul2(mul2(Q, rinv), mul2(rinv, rinv)));
+            const f2 We = mul2(W, e), X = fma2(r2, F2(0.25f), RR);
+            F::add(fr, dx, dy, dz, q, j, p);
+            p.dR[q] = fma2(We, X, p.dR[q]);
+            j.dR = fmaf(We.y, X.y, fmaf(We.x, X.x, j.dR));
+        }
+    }
+    static __device__ __forceinline__ void rotate_acc(J& j, int src) {
+        F::rotate_acc(j, src);
+        j.dR = shfl(j.dR, src);
+    }
+    static __device__ __forceinline__ void fold_i(const PairArgs& A, long long* sa, int lane, const Part& p) {
+        F::template fold<NQ>(sa, lane, p);
+#pragma unroll
+        for (int q = 0; q < 2 * NW; ++q)
+            sa[(q >> 1) * 64 * NQ + 192 + 32 * (q & 1) + lane] += fix(A.en_g * get2(p.dR[q >> 1], q & 1));
+    }
+    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const J& st,
+                                                   const long long* jac = nullptr, int at = 0) {
+        if (j >= n) return;
+        F::flush(A, base + j, st, jac, at);
+        red_add(&A.dR_acc[base + j], fix(A.en_g * st.dR));
+    }
+    static __device__ __forceinline__ float bound(const PairArgs& A, const Slot<EnergyW>&, int) { return A.rep_sigma * A.rep_sigma; }
+    // Soft repulsion of a pair more than one position apart in the chain.
+    static __device__ __forceinline__ void close(const PairArgs& A, const Slot<EnergyW>& S, long long* sa, int i, int j,
+                                                 bool valid, int i0, int jbase) {
+        const float4 xi = S.i4[i], xj = S.j4[j];
+        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz)), rinv = rsqrt_ftz(r2);
+        const int gap = i0 + i - (jbase + j);
+        if (valid && (gap > 1 || gap < -1))
+            F::add_close(sa, S.jac, i, j, 2.0f * A.rep_k * (A.rep_sigma - r2 * rinv) * rinv, dx, dy, dz);
+    }
+};
+
+// --- walking the blocks -------------------------------------------------------------
+// Tiles J0 + (set bits of `mask`) against the W::ATOMS atoms from i0 (a row or
+// a row pair), every block far.  The tile's j data stand in shared memory, the tile twice, so that
+// lane l reads atom (l + k) mod 32 of step k at a fixed offset from its own
+// address: two vector loads a step, free of bank conflicts, in place of six to
+// eight shuffles.  Only the partial sums rotate by shuffles.  A function of
+// its own: inlined into the walk its loop carried a dozen register moves a
+// step (registers of the other paths), 10 to 15 % of its time.  The shuffles
+// at its head tell the compiler that the arguments are the warp's, not the lane's.
+template <class W>
+__device__ __noinline__ void walk_far(const PairArgs& A, int r, int i0, int J0, unsigned mask, int slot) {
+    extern __shared__ __align__(16) unsigned char s_mem[];
+    const int lane = threadIdx.x & 31;
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    r = __shfl_sync(0xffffffffu, r, 0);
+    i0 = __shfl_sync(0xffffffffu, i0, 0);
+    J0 = __shfl_sync(0xffffffffu, J0, 0);
+    mask = __ballot_sync(0xffffffffu, (mask >> lane) & 1u);
+    const int64_t base = A.atom_off[r];
+    const int n = (int)(A.atom_off[r + 1] - base);
+    long long* sa = (long long*)(s_mem + slot);
+    float4* sj = (float4*)(sa + 2 * W::NQ * 64);
+    if (W::ATOMS == 64) sa += ((i0 >> 6) & 1) * 64 * W::NQ;
+    typename W::B* sb = (typename W::B*)(sj + 64);
+    typename W::I is;
+    W::load_i(A, base, n, i0, lane, is);
+    const int next = (lane + 1) & 31;
+    while (mask) {
+        const int j = 32 * (J0 + __ffs(mask) - 1) + lane;
+        mask &= mask - 1;
+        float4 v;
+        typename W::B b;
+        W::load_j(A, base, n, j, v, b);
+        __syncwarp();
+        sj[lane] = sj[32 + lane] = v;
+        sb[lane] = sb[32 + lane] = b;
+        __syncwarp();
+        typename W::J js;
+        typename W::Part p;
+        W::zero(js, p);
+#pragma unroll W::UNROLL
+        for (int k = 0; k < 32; ++k) {
+            W::step(A, is, sj[lane + k], sb[lane + k], js, p);
+            W::rotate_acc(js, next);
+        }
+        W::fold_i(A, sa, lane, p);
+        W::flush_j(A, base, n, j, js);
+    }
+}
+
+// The pairs noted in the lanes' masks (bit k of mx / my: the x / y half's atom
+// against tile atom (lane + k) mod 32), 32 at a time.  Returns their number.
+template <class W>
+__device__ __noinline__ int close_pairs(const PairArgs& A, int slot, int row, unsigned mx, unsigned my, int i0, int jbase) {
+    const int lane = threadIdx.x & 31;
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    row = __shfl_sync(0xffffffffu, row, 0);
+    const Slot<W> S(slot);
+    long long* sa = S.sa + row * 64 * W::NQ;
+    const int own = __popc(mx) + __popc(my);
+    int at = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, at, 31);
+    if (total == 0) return 0;
+#pragma unroll
+    for (int q = 0; q < W::NJ; ++q) S.jac[32 * q + lane] = 0;
+    for (int b0 = 0; b0 < total; b0 += CLOSE_CAP) {
+        int pos = at - own - b0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            unsigned m = h ? my : mx;
+            while (m) {
+                const int k = __ffs(m) - 1;
+                m &= m - 1;
+                if (pos >= 0 && pos < CLOSE_CAP)
+                    S.queue[pos] = (unsigned short)((32 * h + lane) | (((lane + k) & 31) << 6));
+                ++pos;
+            }
+        }
+        __syncwarp();
+        const int cnt = min(CLOSE_CAP, total - b0);
+        for (int e = 0; e < cnt; e += 32) {
+            const int q = S.queue[min(e + lane, cnt - 1)];
+            W::close(A, S, sa, q & 63, q >> 6, e + lane < cnt, i0, jbase);
+        }
+        __syncwarp();
+    }
+    return total;
+}
+
+template <class W, int MODE, bool NEAR>
+__device__ __forceinline__ void near_tile(const PairArgs& A, const typename W::I& is, const Slot<W>& S,
+                                            typename W::J& js, typename W::Part& p, float t, unsigned* mk, int lane) {
+    // a DX block pairs the x half with its own tile: only steps 1 .. 16 carry pairs
+    constexpr int K0 = (MODE == M_DX) ? 1 : 0, K1 = (MODE == M_DX) ? 17 : 32;
+    const int next = (lane + 1) & 31;
+#pragma unroll W::UNROLL
+    for (int k = K0; k < K1; ++k) {
+        W::template step<MODE, NEAR>(A, is, S.j4[lane + k], S.jb[lane + k], js, p, step_mask<MODE>(k, lane), t, 1u << k, mk);
+        W::rotate_acc(js, next);
+    }
+}
+
+// Row K (64 atoms) against tiles J0 + (set bits of `todo`), near or diagonal;
+// t: of lane c the bound below which pairs of column J0 + c are close.
+template <class W, bool CLOSE>
+__device__ __noinline__ void walk_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
+    const int lane = threadIdx.x & 31;
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    r = __shfl_sync(0xffffffffu, r, 0);
+    K = __shfl_sync(0xffffffffu, K, 0);
+    J0 = __shfl_sync(0xffffffffu, J0, 0);
+    todo = __ballot_sync(0xffffffffu, (todo >> lane) & 1u);
+    const int64_t base = A.atom_off[r];
+    const int n = (int)(A.atom_off[r + 1] - base);
+    const Slot<W> S(slot);
+    long long* sa = S.sa + (K & 1) * 64 * W::NQ;
+    typename W::I is;
+    W::load_i(A, base, n, 64 * K, lane, is, S.i4, S.i2);
+    while (todo) {
+        const int c = __ffs(todo) - 1, J = J0 + c;
+        todo &= todo - 1;
+        float4 v;
+        typename W::B b;
+        float2 as;
+        W::load(A, base, n, 32 * J + lane, v, b, as);
+        __syncwarp();
+        S.j4[lane] = S.j4[32 + lane] = v;
+        S.jb[lane] = S.jb[32 + lane] = b;
+        S.ja[lane] = as;
+        __syncwarp();
+        float tc = __shfl_sync(0xffffffffu, t, c);
+        if (!A.boxes) tc = W::bound(A, S, lane);
+        typename W::J js;
+        typename W::Part p;
+        W::zero(js, p);
+        unsigned mk[2] = {0u, 0u};
+        int shift = 0;
+        if (J >= 2 * K + 2) {
+            near_tile<W, M_FULL, CLOSE>(A, is, S, js, p, tc, mk, lane);
+        } else if (J == 2 * K) {
+            near_tile<W, M_DX, CLOSE>(A, is, S, js, p, tc, mk, lane);
+            shift = 17;                    // sums start at atom lane + 1 and leave rotated by 17
+        } else {
+            near_tile<W, M_DY, CLOSE>(A, is, S, js, p, tc, mk, lane);
+        }
+        W::fold_i(A, sa, lane, p);
+        __syncwarp();
+        const int n_close = CLOSE ? close_pairs<W>(A, slot, K & 1, mk[0], mk[1], 64 * K, 32 * J) : 0;
+        const int at = (lane + shift) & 31;
+        W::flush_j(A, base, n, 32 * J + at, js, n_close ? S.jac : nullptr, at);
+    }
+}
+
+// The same row by the general pair code: blocks that straddle a cutoff
+// (EF_STRADDLE), and passes that want energies or dE/dq.
+template <class P, int FLAGS>
+__device__ __noinline__ void walk_general(const PairArgs& A, int r, int K, int J0, unsigned todo, int slot) {
+    extern __shared__ __align__(16) unsigned char s_mem[];
+    const int lane = threadIdx.x & 31, next = (lane + 1) & 31;
+    const int64_t base = A.atom_off[r];
+    const int n = (int)(A.atom_off[r + 1] - base), nb = (n + 31) >> 5;
+    long long* sa = (long long*)(s_mem + slot) + (K & 1) * 64 * P::NQ;
     typename P::IState is;
     P::load_i(A, base, n, 64 * K, lane, is);
-    const int next = (lane + 1) & 31;
-    // EF_CUT: straddling blocks run the pair code with EF_STRADDLE.  The task
-    // list is the block neighbour list (k_block_list: in-range blocks only),
-    // or, without tile boxes, every block, each counted as straddling.
-    constexpr int FS = (FLAGS & EF_CUT) ? (FLAGS | EF_STRADDLE) : FLAGS;
-    for (int c = 0; c < cnt; ++c) {
-        const bool dx = (J == 2 * K);          // see run_tile: entry / exit rotation of a DX block
+    while (todo) {
+        const int J = J0 + __ffs(todo) - 1;
+        todo &= todo - 1;
+        const bool dx = (J == 2 * K);      // see run_tile: entry / exit rotation of a DX block
         typename P::JState js;
         P::load_j(A, base, n, 32 * J + ((lane + (dx ? 1 : 0)) & 31), js);
         typename P::Part ip;
         ip.zero();
         const BlockInfo bi = block_info<P>(A, r, K, J, nb);
-        const bool straddle = (FLAGS & EF_CUT) && bi.straddle;
         if (J >= 2 * K + 2) {
-            if (bi.far && !straddle) run_tile<P, FLAGS, M_FULL, true>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
-            else if (straddle) run_tile<P, FS, M_FULL, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
+            if (!(FLAGS & EF_STRADDLE) && bi.far) run_tile<P, FLAGS, M_FULL, true>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
             else run_tile<P, FLAGS, M_FULL, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
-        } else if (J == 2 * K) {
-            if (straddle) run_tile<P, FS, M_DX, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
-            else run_tile<P, FLAGS, M_DX, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
+        } else if (dx) {
+            run_tile<P, FLAGS, M_DX, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
         } else {
-            if (straddle) run_tile<P, FS, M_DY, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
-            else run_tile<P, FLAGS, M_DY, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
+            run_tile<P, FLAGS, M_DY, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
         }
         P::fold_i(is, sa, lane, ip);
         P::flush_j(A, base, n, 32 * J + ((lane + (dx ? 17 : 0)) & 31), js);
-        if (c + 1 < cnt && ++J == nb) {
-            P::flush_i(A, r, base, n, 64 * K, lane, is, sa);
+    }
+    P::flush_sums(A, r, lane, is);
+}
+
+// Form of a block (see above) from the bounds of its boxes.
+template <class P, int FLAGS>
+__device__ __forceinline__ int row_tier(const PairArgs& A, const BoxPair& b) {
+    if (P::RADIUS_CUT) {
+        const float as = b.amax + b.smax, s2 = b.smax * b.smax;
+        if (b.rmin2 < as * as || s2 > GB_POLY_YFAR * b.rmin2) return 0;
+        const float y3 = P::CHAIN ? GB_Y_H3 : GB_Y_G3, y2 = P::CHAIN ? GB_Y_H2 : GB_Y_G2;
+        return s2 <= y2 * b.rmin2 ? 3 : (s2 <= y3 * b.rmin2 ? 2 : 1);
+    }
+    return (!(FLAGS & EF_REP) || b.rmin2 >= A.rep_sigma * A.rep_sigma) ? 1 : 0;
+}
+
+// Far tiles of a row (NW 1) or a row pair (NW 2).
+template <class P, int FLAGS, int NW>
+__device__ __forceinline__ void run_far(int tier, const PairArgs& A, int r, int i0, int J0, unsigned mask, int slot) {
+    if constexpr (!P::RADIUS_CUT) {
+        walk_far<EnergyW<NW, FLAGS & EF_SALT>>(A, r, i0, J0, mask, slot);
+    } else if constexpr (P::CHAIN) {
+        if (NW == 2 && tier == 3) walk_far<ChainU<2, 2>>(A, r, i0, J0, mask, slot);
+        else if (tier >= 2) walk_far<ChainU<NW, 3>>(A, r, i0, J0, mask, slot);
+        else walk_far<ChainY<NW>>(A, r, i0, J0, mask, slot);
+    } else {
+        if (NW == 2 && tier == 3) walk_far<BornU<2, 2>>(A, r, i0, J0, mask, slot);
+        else if (tier >= 2) walk_far<BornU<NW, 3>>(A, r, i0, J0, mask, slot);
+        else walk_far<BornY<NW>>(A, r, i0, J0, mask, slot);
+    }
+}
+template <class P, int FLAGS>
+__device__ __forceinline__ void run_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
+    if constexpr (!P::RADIUS_CUT) walk_near<EnergyW<1, FLAGS & EF_SALT>, (FLAGS & EF_REP) != 0>(A, r, K, J0, todo, t, slot);
+    else if constexpr (P::CHAIN) walk_near<ChainY<1>, true>(A, r, K, J0, todo, t, slot);
+    else walk_near<BornY<1>, true>(A, r, K, J0, todo, t, slot);
+}
+
+// Work of replica r is walked as row pairs P = 0 .. ceil(nb/4) - 1 (nb tiles
+// of 32 atoms; 128 atoms each, rows K = 2P and 2P + 1), each over the tiles
+// (columns) J = 4P .. nb-1.  A warp task is (replica, 4P + rows, J, columns):
+// rows is 1 or 2 for one row of the pair alone, 3 for both.  Columns where
+// both rows are far (and inside every cutoff) are evaluated 128 x 32 by
+// the task that holds row 0, the others row by row in 64 x 32 blocks.  Replicas
+// of up to SMALL_TILES tiles run every block 64 x 32: their pass ends with the
+// slowest warps, and half the block halves what the last ones still do.  Every
+// choice depends on the replica and the block alone, so that results do not
+// depend on how the work is cut or on what else is in the batch.  SMALL: the
+// kernel for batches of small replicas alone (no 128 x 32 code, fewer registers).
+//
+// The tile boxes of 32 columns are classified at once, one column a lane.
+// slot is the byte offset of the warp's shared memory (see Slot).  Loads of
+// data that kernels rewrite (coordinates, radii, chain factors, boxes) go
+// through L2 (ld.global.cg): a persistent launch reads them again after other
+// SMs changed them, and L1 is not coherent.
+template <class P, int FLAGS, bool SMALL = false>
+__device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, int slot, int lane) {
+    extern __shared__ __align__(16) unsigned char s_mem[];
+    long long* sa = (long long*)(s_mem + slot);
 #pragma unroll
-            for (int q = 0; q < 2 * P::NQ; ++q) sa[32 * q + lane] = 0;
-            if (++K == nk) {
-                do {
-                    ++r;
-                    base = A.atom_off[r];
-                    n = (int)(A.atom_off[r + 1] - base);
-                    nb = (n + 31) >> 5;
-                } while (nb == 0);
-                nk = (nb + 1) >> 1;
-                K = 0;
+    for (int q = 0; q < 4 * P::NQ; ++q) sa[32 * q + lane] = 0;
+    __syncwarp();
+    // energies and dE/dq have the general pair code alone, blocks that
+    // straddle a cutoff too (without tile boxes every block counts as one)
+    constexpr bool GENERAL = !P::RADIUS_CUT && (FLAGS & (EF_ENERGY | EF_PHI)) != 0;
+    constexpr bool CUT = (FLAGS & EF_CUT) != 0;
+    const int r = t.x, PR = t.y >> 2, sel = t.y & 3;
+    const int64_t base = A.atom_off[r];
+    const int n = (int)(A.atom_off[r + 1] - base);
+    const int nb = (n + 31) >> 5;
+    unsigned used = 0;
+    for (int s0 = 0; s0 < t.w; s0 += 32) {
+        const int J0 = t.z + s0, m = min(32, t.w - s0), J = J0 + lane;
+        int tier[2] = {0, 0};
+        bool in[2] = {true, true}, straddle[2] = {CUT, CUT};
+        float bound[2] = {0.0f, 0.0f};
+        if (A.boxes && lane < m) {
+            const int t0 = A.tile_off[r];
+            const float4 jl = __ldcg(&A.boxes[2 * (t0 + J)]), jh = __ldcg(&A.boxes[2 * (t0 + J) + 1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (4 * PR + 2 * h >= nb) continue;
+                float4 ih;
+                const float4 il = row_box_lo(A, t0, 2 * PR + h, nb, &ih);
+                const BoxPair b = box_pair(il, ih, jl, jh);
+                tier[h] = row_tier<P, FLAGS>(A, b);
+                bound[h] = P::RADIUS_CUT ? close_bound(b.amax, b.smax) : A.rep_sigma * A.rep_sigma;
+                if (CUT) cut_class(A, P::RADIUS_CUT, b, in[h], straddle[h]);
             }
-            J = 2 * K;
-            P::load_i(A, base, n, 64 * K, lane, is);
+        }
+        const unsigned all = m == 32 ? 0xffffffffu : (1u << m) - 1u;
+        unsigned wide = 0;
+        if (!GENERAL && !SMALL && nb > SMALL_TILES) {
+            const int both = (J >= 4 * PR + 4 && (!CUT || (in[0] && in[1] && !straddle[0] && !straddle[1])))
+                                 ? min(tier[0], tier[1]) : 0;
+#pragma unroll
+            for (int k = P::RADIUS_CUT ? 3 : 1; k > 0; --k) {
+                const unsigned w = __ballot_sync(0xffffffffu, both == k) & all;
+                if (w && (sel & 1)) run_far<P, FLAGS, 2>(k, A, r, 128 * PR, J0, w, slot);
+                wide |= w;
+            }
+            if (wide && (sel & 1)) used |= 3;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int K = 2 * PR + h;
+            unsigned todo = all & ~wide;
+            if (CUT) todo &= __ballot_sync(0xffffffffu, in[h]);
+            if (J0 < 2 * K) todo &= ~((1u << (2 * K - J0)) - 1u);      // tiles before the row's diagonal
+            if (!((sel >> h) & 1) || 2 * K >= nb || !todo) continue;
+            used |= 1u << h;
+            const unsigned st = CUT ? todo & __ballot_sync(0xffffffffu, straddle[h]) : 0u, rest = todo & ~st;
+            if constexpr (CUT) {
+                if (st) walk_general<P, FLAGS | EF_STRADDLE>(A, r, K, J0, st, slot);
+            }
+            if constexpr (GENERAL) {
+                if (rest) walk_general<P, FLAGS>(A, r, K, J0, rest, slot);
+            } else {
+                const bool diag = J < 2 * K + 2;
+                const unsigned near = rest & __ballot_sync(0xffffffffu, diag || tier[h] == 0);
+                const unsigned far1 = rest & __ballot_sync(0xffffffffu, !diag && tier[h] == 1), far2 = rest & ~(near | far1);
+                if (near) run_near<P, FLAGS>(A, r, K, J0, near, bound[h], slot);
+                if (far1) run_far<P, FLAGS, 1>(1, A, r, 64 * K, J0, far1, slot);
+                if (far2) run_far<P, FLAGS, 1>(2, A, r, 64 * K, J0, far2, slot);
+            }
         }
     }
-    P::flush_i(A, r, base, n, 64 * K, lane, is, sa);
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if ((used >> h) & 1) P::flush_i(A, base, n, 128 * PR + 64 * h, lane, sa + h * 64 * P::NQ);
 }
 
 
@@ -1074,14 +1851,15 @@ __device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, long 
 // One warp per task.  MINB = 1 leaves the register count to the compiler;
 // MINB = 3 or 4 caps it so that three or four 256-thread blocks fit on an SM
 // (more warps, some spills).
-template <class P, int FLAGS, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_pairs(PairArgs A, const int4* __restrict__ tasks, int n_tasks) {
+template <class P, int FLAGS, int MINB, bool SMALL>
+__global__ void __launch_bounds__(256, MINB) k_pairs(const __grid_constant__ PairArgs A, const int4* __restrict__ tasks, int n_tasks) {
     pdl_enter();
-    extern __shared__ long long s_acc[];
     const int lane = threadIdx.x & 31;
-    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    // the shuffle tells the compiler that the task is the same for the whole
+    // warp: uniform loops and addresses, 3 to 5 % of a distant block
+    const int w = __shfl_sync(0xffffffffu, (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), 0);
     if (w >= n_tasks) return;
-    walk_task<P, FLAGS>(A, tasks[w], s_acc + (threadIdx.x >> 5) * P::NQ * 64, lane);
+    walk_task<P, FLAGS, SMALL>(A, tasks[w], (threadIdx.x >> 5) * WARP_SMEM<P>, lane);
 }
 
 // The same pass over a task list built on the device (cutoff passes: the
@@ -1089,35 +1867,37 @@ __global__ void __launch_bounds__(256, MINB) k_pairs(PairArgs A, const int4* __r
 // and warps take tasks one at a time from the queue head ctr[head_idx] until
 // it runs dry, so the grid only needs to fill the GPU.
 template <class P, int FLAGS, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_pairs_dyn(PairArgs A, const int4* __restrict__ tasks, int* ctr,
+__global__ void __launch_bounds__(256, MINB) k_pairs_dyn(const __grid_constant__ PairArgs A, const int4* __restrict__ tasks, int* ctr,
                                                          int count_idx, int head_idx) {
     pdl_enter();
-    extern __shared__ long long s_acc[];
-    const int lane = threadIdx.x & 31;
-    long long* sa = s_acc + (threadIdx.x >> 5) * P::NQ * 64;
+    const int lane = threadIdx.x & 31, slot = (threadIdx.x >> 5) * WARP_SMEM<P>;
     const int n_tasks = __ldcg(&ctr[count_idx]);
     for (;;) {
         int w = 0;
         if (lane == 0) w = atomicAdd(&ctr[head_idx], 1);
         w = __shfl_sync(0xffffffffu, w, 0);
         if (w >= n_tasks) break;
-        walk_task<P, FLAGS>(A, __ldcg(&tasks[w]), sa, lane);
+        walk_task<P, FLAGS>(A, __ldcg(&tasks[w]), slot, lane);
     }
 }
 
-// Launch of pass policy P over a task list; MAXCAP limits the register caps
-// instantiated (a larger cap request takes the largest one available).
-template <class P, int FLAGS, int MAXCAP = 4>
+// Launch of pass policy P over a task list.
+template <class P, int FLAGS, bool SMALL>
+cudaError_t launch_pass_cap(const PairArgs& a, const TaskList& t, int cap, int wpb, cudaStream_t s) {
+    wpb = fit_warps<P>(wpb);
+    const size_t smem = (size_t)wpb * WARP_SMEM<P>;
+    const dim3 g((t.n_tasks + wpb - 1) / wpb), b(32 * wpb);
+    if (cap >= 4) return launch_pdl(k_pairs<P, FLAGS, 4, SMALL>, g, b, smem, s, a, t.d_tasks, t.n_tasks);
+    if (cap >= 3) return launch_pdl(k_pairs<P, FLAGS, 3, SMALL>, g, b, smem, s, a, t.d_tasks, t.n_tasks);
+    return launch_pdl(k_pairs<P, FLAGS, 2, SMALL>, g, b, smem, s, a, t.d_tasks, t.n_tasks);
+}
+template <class P, int FLAGS>
 cudaError_t launch_pass(const PairArgs& a, const TaskList& t, int cap, int wpb, cudaStream_t s) {
     if (t.n_tasks == 0) return cudaSuccess;
-    const int blocks = (t.n_tasks + wpb - 1) / wpb;
-    const size_t smem = (size_t)wpb * P::NQ * 64 * sizeof(long long);
-    const dim3 g(blocks), b(32 * wpb);
-    if constexpr (MAXCAP >= 4) {
-        if (cap >= 4) return launch_pdl(k_pairs<P, FLAGS, 4>, g, b, smem, s, a, t.d_tasks, t.n_tasks);
+    if constexpr (P::RADIUS_CUT || !(FLAGS & (EF_ENERGY | EF_PHI))) {
+        if (t.small) return launch_pass_cap<P, FLAGS, true>(a, t, cap, wpb, s);
     }
-    if (cap >= 3) return launch_pdl(k_pairs<P, FLAGS, 3>, g, b, smem, s, a, t.d_tasks, t.n_tasks);
-    return launch_pdl(k_pairs<P, FLAGS, 1>, g, b, smem, s, a, t.d_tasks, t.n_tasks);
+    return launch_pass_cap<P, FLAGS, false>(a, t, cap, wpb, s);
 }
 
 // Bounding boxes of every 32-atom tile (one warp per tile): lo.xyz with the

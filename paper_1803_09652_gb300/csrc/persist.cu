@@ -31,7 +31,8 @@
 namespace gbk {
 
 constexpr int PERSIST_THREADS = 128;
-constexpr int PERSIST_NQ = Energy::NQ;   // largest i-side accumulator slot of the three passes
+constexpr int PERSIST_SMEM = WARP_SMEM<Energy>;   // the largest of the three passes' slots
+static_assert(PERSIST_SMEM >= WARP_SMEM<Chain> && PERSIST_SMEM >= WARP_SMEM<Born>, "slot");
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
@@ -116,11 +117,10 @@ __device__ __forceinline__ void atoms_chain_bonds(const PersistArgs& P, int r, i
 }
 
 template <int REP>
-__global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(PersistArgs P) {
-    extern __shared__ long long s_acc[];
+__global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(const __grid_constant__ PersistArgs P) {
     constexpr int EFL = REP ? EF_REP : 0;
     const int lane = threadIdx.x & 31;
-    long long* sa = s_acc + (threadIdx.x >> 5) * PERSIST_NQ * 64;
+    const int slot = (threadIdx.x >> 5) * PERSIST_SMEM;
     const unsigned per_step = (unsigned)P.phase_base[6];
     const unsigned total = per_step * (unsigned)P.nsteps + (unsigned)P.phase_base[1];
     const u64 step0 = __ldcg(&P.md.ctr[0]) + (u64)P.step0;
@@ -154,16 +154,16 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(PersistArgs P
         if (!ok) break;
         switch (p) {
             case 0: tile_halfsteps(P, r, u, lane, s > 0, s < P.nsteps, step0 + (u64)s + 1); break;
-            case 1: walk_task<Born, 0>(P.pa, P.tasks[P.task_off[r] + u], sa, lane); break;
+            case 1: walk_task<Born, 0>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
             case 2: {
                 const int64_t base = P.pa.atom_off[r];
                 const int i = 32 * u + lane;
                 if (i < (int)(P.pa.atom_off[r + 1] - base)) born_finalize_atom(P.aa, base + i, P.R_out);
                 break;
             }
-            case 3: walk_task<EnergyF<EFL>, EFL>(P.pa, P.tasks[P.task_off[r] + u], sa, lane); break;
+            case 3: walk_task<EnergyF<EFL>, EFL>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
             case 4: atoms_chain_bonds(P, r, u, lane); break;
-            default: walk_task<Chain, 0>(P.pa, P.tasks[P.task_off[r] + u], sa, lane); break;
+            default: walk_task<Chain, 0>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
         }
         __threadfence();
         __syncwarp();
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(PersistArgs P
     }
 }
 
-size_t persist_smem() { return (size_t)(PERSIST_THREADS / 32) * PERSIST_NQ * 64 * sizeof(long long); }
+size_t persist_smem() { return (size_t)(PERSIST_THREADS / 32) * PERSIST_SMEM; }
 
 cudaError_t persist_occupancy(int rep, int* blocks_per_sm) {
     const size_t smem = persist_smem();

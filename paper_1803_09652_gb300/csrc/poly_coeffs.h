@@ -30,6 +30,33 @@ __device__ __forceinline__ float gb_poly_hf(float y) {
 __device__ __forceinline__ float2 gb_poly_hf2(float2 y) {
     return __ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(make_float2(1.854454994e+01f, 1.854454994e+01f), y, make_float2(1.023153305e+01f, 1.023153305e+01f)), y, make_float2(8.925169945e+00f, 8.925169945e+00f)), y, make_float2(6.856277943e+00f, 6.856277943e+00f)), y, make_float2(4.800007343e+00f, 4.800007343e+00f)), y, make_float2(2.666666746e+00f, 2.666666746e+00f));
 }
+#define GB_POLY_YNEAR 0.20000000f
+/* gn(y) on [0, 0.2], degree 6, max relative error in FP32 Horner 8.55e-08 */
+__device__ __forceinline__ float gb_poly_gn(float y) {
+    return fmaf(fmaf(fmaf(fmaf(fmaf(fmaf(2.006710768e+00f, y, 5.837699175e-01f), y, 9.585292339e-01f), y, 8.852983713e-01f), y, 8.572651148e-01f), y, 7.999984622e-01f), y, 6.666666865e-01f);
+}
+__device__ __forceinline__ float2 gb_poly_gn2(float2 y) {
+    return __ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(make_float2(2.006710768e+00f, 2.006710768e+00f), y, make_float2(5.837699175e-01f, 5.837699175e-01f)), y, make_float2(9.585292339e-01f, 9.585292339e-01f)), y, make_float2(8.852983713e-01f, 8.852983713e-01f)), y, make_float2(8.572651148e-01f, 8.572651148e-01f)), y, make_float2(7.999984622e-01f, 7.999984622e-01f)), y, make_float2(6.666666865e-01f, 6.666666865e-01f));
+}
+/* hn(y) on [0, 0.2], degree 6, max relative error in FP32 Horner 8.85e-08 */
+__device__ __forceinline__ float gb_poly_hn(float y) {
+    return fmaf(fmaf(fmaf(fmaf(fmaf(fmaf(3.545024109e+01f, y, 6.343571663e+00f), y, 1.187423325e+01f), y, 8.818530083e+00f), y, 6.859543324e+00f), y, 4.799969673e+00f), y, 2.666666746e+00f);
+}
+__device__ __forceinline__ float2 gb_poly_hn2(float2 y) {
+    return __ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(__ffma2_rn(make_float2(3.545024109e+01f, 3.545024109e+01f), y, make_float2(6.343571663e+00f, 6.343571663e+00f)), y, make_float2(1.187423325e+01f, 1.187423325e+01f)), y, make_float2(8.818530083e+00f, 8.818530083e+00f)), y, make_float2(6.859543324e+00f, 6.859543324e+00f)), y, make_float2(4.799969673e+00f, 4.799969673e+00f)), y, make_float2(2.666666746e+00f, 2.666666746e+00f));
+}
+/* g(y) on [0, 0.025], degree 3, relative error of the coefficients 3.83e-08 */
+#define GB_Y_G3 0.02500000f
+#define GB_G3 {6.666666865e-01f, 8.000037074e-01f, 8.563990593e-01f, 9.359787107e-01f}
+/* g(y) on [0, 0.009], degree 2, relative error of the coefficients 3.19e-08 */
+#define GB_Y_G2 0.00900000f
+#define GB_G2 {6.666666865e-01f, 7.999589443e-01f, 8.692682981e-01f}
+/* h(y) on [0, 0.0185], degree 3, relative error of the coefficients 3.73e-08 */
+#define GB_Y_H3 0.01850000f
+#define GB_H3 {2.666666746e+00f, 4.800017834e+00f, 6.852286339e+00f, 9.305003166e+00f}
+/* h(y) on [0, 0.006], degree 2, relative error of the coefficients 2.98e-08 */
+#define GB_Y_H2 0.00600000f
+#define GB_H2 {2.666666746e+00f, 4.799818039e+00f, 6.937810421e+00f}
 #define GB_POLY_ZJ 0.50000000f
 /* q(y) on [0, 0.5], degree 9, max relative error in FP32 Horner 1.19e-07 */
 __device__ __forceinline__ float gb_poly_q(float y) {
