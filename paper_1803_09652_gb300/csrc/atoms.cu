@@ -253,12 +253,80 @@ __device__ __forceinline__ float mc_self_term(float Rk, float tke, float kc, flo
     return -t / Rk;
 }
 
+// Sum of FP32 terms to about 2^-40 of its size without FP64, which this GPU
+// issues at 1/64 of the FP32 rate: s carries the rounded sum and c the exact
+// rounding errors of its additions (Knuth's two-sum).
+struct Sum2 {
+    float s = 0.0f, c = 0.0f;
+    __device__ __forceinline__ void add(float x, float low = 0.0f) {
+        const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+        c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)) + low;
+        s = t;
+    }
+    // + (h + l) a, with the product's rounding error
+    __device__ __forceinline__ void add_product(float h, float l, float a) {
+        const float p = __fmul_rn(h, a);
+        add(p, fmaf(l, a, fmaf(h, a, -p)));
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
+// Rows phi of `count` site atoms (replica-local index idx(k)) over the slice
+// j0 .. j1 of the replica's atoms, by one block of 8 warps: out[k].
+// A lane owns a site atom and walks the slice's atoms in shared memory (read
+// by all lanes at once), so that no reduction over lanes is left; the warps
+// share the slice of a 32-atom group of site atoms (two of them, more when
+// there are fewer than eight groups), so that their number divides the work.
+// Bound by the pair term's FP32 and MUFU instructions, about 30 a term.  As
+// one warp a site atom with FP64 sums per lane and an FP64 shuffle tree, the
+// FP64 pipe took six times as long as the terms: 530 us for 4 x 25000 atoms
+// and their 620 site atoms a replica.
+template <class Idx>
+__device__ __forceinline__ void mc_rows_slice(const MCArgs& A, int64_t base, int j0, int j1, int count, Idx idx,
+                                              double* out) {
+    __shared__ float4 s_x[MC_CHUNK];
+    __shared__ float2 s_R[MC_CHUNK];
+    __shared__ double s_part[2 * SWEEP_MAX_SITE_ATOMS / 32][32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nj = j1 - j0;
+    for (int j = tid; j < nj; j += blockDim.x) {
+        s_x[j] = A.xyzq[base + j0 + j];
+        s_R[j] = mc_Rh(A, base + j0 + j);
+    }
+    __syncthreads();
+    const float tke = (float)A.tau_ke, kc = (float)A.kc, keo = (float)A.ke_out, kap = (float)A.kappa;
+    const int groups = (count + 31) >> 5;
+    const int share = groups >= 8 ? 2 : max(2, 8 / groups);    // parts of a group's slice
+    const int seg = (nj + share - 1) / share;
+    for (int u = wid; u < groups * share; u += 8) {
+        const int k = 32 * (u / share) + lane, part = u % share;
+        const int lk = idx(min(k, count - 1));
+        const float4 xk = A.xyzq[base + lk];
+        const float2 Rk = mc_Rh(A, base + lk);
+        const float self = mc_self_term(Rk.x, tke, kc, keo, kap);
+        Sum2 sum;
+        const int end = min(nj, (part + 1) * seg);
+#pragma unroll 4
+        for (int j = part * seg; j < end; ++j) {
+            const float4 xj = s_x[j];
+            const float term = mc_pair_term(xk, Rk, xj, s_R[j], tke, kc, keo, kap, A.cut2);
+            sum.add(__fmul_rn(xj.w, j0 + j == lk ? self : term));    // rounded: not fused into the sum
+        }
+        s_part[u][lane] = sum.value();
+    }
+    __syncthreads();
+    for (int k = tid; k < count; k += blockDim.x) {
+        double v = 0.0;
+        for (int part = 0; part < share; ++part) v += s_part[(k >> 5) * share + part][k & 31];
+        out[k] = v;
+    }
+}
+
 __global__ void __launch_bounds__(256) k_mc_rows(MCArgs A) {
     pdl_enter();
     __shared__ MCPick s_pick;
     const int r = blockIdx.y, part = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    if (tid == 0) s_pick = mc_pick(A, r);
+    if (threadIdx.x == 0) s_pick = mc_pick(A, r);
     __syncthreads();
     const int site = s_pick.site;
     if (site < 0) return;
@@ -269,24 +337,9 @@ __global__ void __launch_bounds__(256) k_mc_rows(MCArgs A) {
     const int n = (int)(A.atom_off[r + 1] - base);
     if (!mc_site_ok(A, s_pick, a0, na, n)) return;
     const int j0 = part * MC_CHUNK, j1 = min(n, j0 + MC_CHUNK);
-    const float tke = (float)A.tau_ke, kc = (float)A.kc, keo = (float)A.ke_out, kap = (float)A.kappa;
-    double* out = A.phi_part + ((size_t)r * A.n_parts + part) * MC_MAX_SITE_ATOMS;
-    for (int k = wid; k < na; k += nw) {
-        const int lk = A.site_atom_idx[a0 + k];
-        const int64_t gk = base + lk;
-        const float4 xk = A.xyzq[gk];
-        const float2 Rk = mc_Rh(A, gk);
-        double acc = 0.0;
-        for (int j = j0 + lane; j < j1; j += 32) {
-            const int64_t gj = base + j;
-            const float4 xj = A.xyzq[gj];
-            const float term = (j == lk) ? mc_self_term(Rk.x, tke, kc, keo, kap) : mc_pair_term(xk, Rk, xj, mc_Rh(A, gj), tke, kc, keo, kap, A.cut2);
-            acc += (double)(xj.w * term);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) out[k] = acc;
-    }
+    if (j0 >= n) return;
+    mc_rows_slice(A, base, j0, j1, na, [&](int k) { return A.site_atom_idx[a0 + k]; },
+                  A.phi_part + ((size_t)r * A.n_parts + part) * MC_MAX_SITE_ATOMS);
 }
 
 __global__ void __launch_bounds__(256) k_mc_decide(MCArgs A) {
@@ -383,37 +436,53 @@ struct SweepList {
 };
 
 // Built by the whole block; false (for every thread) when replica r's sites
-// of the kind exceed the limits.
+// of the kind exceed the limits.  The first warp scans 32 sites at a time and
+// a warp takes a site's atoms: one thread walking the tables paid their
+// latency site by site, about 40 us for 40 sites.
 __device__ bool sweep_list(const MCArgs& A, int r, SweepList& L) {
     __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        int ns = 0, na = 0, ok = 1;
-        for (int s = A.site_off[r]; s < A.site_off[r + 1] && ok; ++s) {
-            if (A.site_kind[s] != A.kind) continue;
-            const int n_s = A.site_atom_off[s + 1] - A.site_atom_off[s];
-            if (ns >= SWEEP_MAX_SITES || na + n_s > SWEEP_MAX_SITE_ATOMS || n_s > MC_MAX_SITE_ATOMS || n_s < 1) {
-                ok = 0;
-                break;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid == 0) {
+        int ns = 0, na = 0;
+        bool ok = true;
+        const int end = A.site_off[r + 1];
+        for (int s0 = A.site_off[r]; s0 < end && ok; s0 += 32) {
+            const int s = s0 + lane;
+            const bool mine = s < end && A.site_kind[s] == A.kind;
+            const int n_s = mine ? A.site_atom_off[s + 1] - A.site_atom_off[s] : 0;
+            const unsigned m = __ballot_sync(0xffffffffu, mine);
+            ok = !__any_sync(0xffffffffu, mine && (n_s > MC_MAX_SITE_ATOMS || n_s < 1));
+            int at = n_s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += v;
             }
-            L.site[ns] = s;
-            L.first[ns] = na;
-            ++ns;
-            na += n_s;
+            const int k = ns + __popc(m & ((1u << lane) - 1u)), first = na + at - n_s;
+            ns += __popc(m);
+            na += __shfl_sync(0xffffffffu, at, 31);
+            ok = ok && ns <= SWEEP_MAX_SITES && na <= SWEEP_MAX_SITE_ATOMS;
+            if (ok && mine) {
+                L.site[k] = s;
+                L.first[k] = first;
+            }
         }
-        L.n_sites = ns;
-        L.n_atoms = na;
-        L.first[ns] = na;
-        s_ok = ok;
-        if (!ok && A.err) atomicCAS(A.err, 0, GB_ERR_INVALID_ARG);
+        if (lane == 0) {
+            s_ok = ok;
+            L.n_sites = ok ? ns : 0;
+            L.n_atoms = ok ? na : 0;
+            if (ok) L.first[ns] = na;
+            if (!ok && A.err) atomicCAS(A.err, 0, GB_ERR_INVALID_ARG);
+        }
     }
     __syncthreads();
     if (!s_ok) return false;
     // the table checks of mc_site_ok for every listed site
     const int n = (int)(A.atom_off[r + 1] - A.atom_off[r]);
     bool bad = false;
-    for (int k = 0; k < L.n_sites; ++k) {
+    for (int k = wid; k < L.n_sites; k += blockDim.x >> 5) {
         const int a0 = A.site_atom_off[L.site[k]];
-        for (int a = threadIdx.x; a < L.first[k + 1] - L.first[k]; a += blockDim.x) {
+        for (int a = lane; a < L.first[k + 1] - L.first[k]; a += 32) {
             const int idx = A.site_atom_idx[a0 + a];
             bad |= idx < 0 || idx >= n;
             L.atom[L.first[k] + a] = idx;
@@ -435,41 +504,37 @@ __global__ void __launch_bounds__(256) k_sweep_rows(MCArgs A) {
     pdl_enter();
     __shared__ SweepList L;
     const int r = blockIdx.y, part = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    if (!sweep_list(A, r, L) || L.n_sites == 0) return;
     const int64_t base = A.atom_off[r];
     const int n = (int)(A.atom_off[r + 1] - base);
     const int j0 = part * MC_CHUNK, j1 = min(n, j0 + MC_CHUNK);
-    const float tke = (float)A.tau_ke, kc = (float)A.kc, keo = (float)A.ke_out, kap = (float)A.kappa;
-    double* out = A.phi_part + ((size_t)r * A.n_parts + part) * SWEEP_MAX_SITE_ATOMS;
-    for (int k = wid; k < L.n_atoms; k += nw) {
-        const int lk = L.atom[k];
-        const int64_t gk = base + lk;
-        const float4 xk = A.xyzq[gk];
-        const float2 Rk = mc_Rh(A, gk);
-        double acc = 0.0;
-        for (int j = j0 + lane; j < j1; j += 32) {
-            const int64_t gj = base + j;
-            const float4 xj = A.xyzq[gj];
-            const float term = (j == lk) ? mc_self_term(Rk.x, tke, kc, keo, kap) : mc_pair_term(xk, Rk, xj, mc_Rh(A, gj), tke, kc, keo, kap, A.cut2);
-            acc += (double)(xj.w * term);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) out[k] = acc;
-    }
+    if (j0 >= n) return;
+    if (!sweep_list(A, r, L) || L.n_sites == 0) return;
+    mc_rows_slice(A, base, j0, j1, L.n_atoms, [&](int k) { return L.atom[k]; },
+                  A.phi_part + ((size_t)r * A.n_parts + part) * SWEEP_MAX_SITE_ATOMS);
 }
 
-__global__ void __launch_bounds__(256) k_sweep_decide(MCArgs A) {
+// One block a replica; the visits follow one another, so what a visit waits
+// for is kept short: the numbers of all visits are drawn at once beforehand
+// (their order, proposals and Metropolis thresholds -kT ln u depend on no
+// decision), coordinates, radii and charges of the listed atoms stand in shared
+// memory, sums over the rows use Sum2 instead of FP64, and an accepted move
+// updates only the rows of sites still to be visited.
+constexpr int SWEEP_THREADS = 1024;
+__global__ void __launch_bounds__(SWEEP_THREADS) k_sweep_decide(MCArgs A) {
     pdl_enter();
     __shared__ SweepList L;
     __shared__ double s_phi[SWEEP_MAX_SITE_ATOMS];
-    __shared__ double s_dq[MC_MAX_SITE_ATOMS];
-    __shared__ int s_order[SWEEP_MAX_SITES];
-    __shared__ double sh[32];
-    __shared__ int s_li, s_site, s_nxt, s_acc;
+    __shared__ float4 s_x[SWEEP_MAX_SITE_ATOMS];
+    __shared__ float2 s_R[SWEEP_MAX_SITE_ATOMS];
+    __shared__ double s_u[SWEEP_MAX_SITES];
+    __shared__ unsigned short s_order[SWEEP_MAX_SITES];
+    __shared__ unsigned s_w0[SWEEP_MAX_SITES], s_w1[SWEEP_MAX_SITES];
+    __shared__ float2 s_dq[MC_MAX_SITE_ATOMS];
+    __shared__ float s_qnew[MC_MAX_SITE_ATOMS];
+    __shared__ double s_sum[SWEEP_THREADS / 32];
+    __shared__ int s_acc;
     const int r = blockIdx.x;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     // every site of the replica starts as "not visited"
     for (int s = A.site_off[r] + tid; s < A.site_off[r + 1]; s += blockDim.x) {
         if (A.dG_out) A.dG_out[s] = 0.0;
@@ -480,82 +545,110 @@ __global__ void __launch_bounds__(256) k_sweep_decide(MCArgs A) {
     const int n = (int)(A.atom_off[r + 1] - base);
     const int n_parts_r = (n + MC_CHUNK - 1) / MC_CHUNK;
     for (int k = tid; k < L.n_atoms; k += blockDim.x) {
+        const double* part = A.phi_part + (size_t)r * A.n_parts * SWEEP_MAX_SITE_ATOMS + k;
         double phi = 0.0;
-        for (int p = 0; p < n_parts_r; ++p)
-            phi += A.phi_part[((size_t)r * A.n_parts + p) * SWEEP_MAX_SITE_ATOMS + k];
+#pragma unroll 16
+        for (int p = 0; p < n_parts_r; ++p) phi += part[(size_t)p * SWEEP_MAX_SITE_ATOMS];
         s_phi[k] = phi;
+        s_x[k] = A.xyzq[base + L.atom[k]];
+        s_R[k] = mc_Rh(A, base + L.atom[k]);
     }
-    for (int k = tid; k < L.n_sites; k += blockDim.x) s_order[k] = k;
-    __syncthreads();
     const u64 step = (A.ctr ? A.ctr[0] : 0) + A.step;
-    const float tke = (float)A.tau_ke, kc = (float)A.kc, keo = (float)A.ke_out, kap = (float)A.kappa;
-    double u = 0.0;
-    int cur = 0;
-    for (int i = 0; i < L.n_sites; ++i) {
-        if (tid == 0) {
-            const Philox4 w = philox4x64(A.rep_base + (u64)r, step, 5 + (u64)A.kind, (u64)i, A.seed, 0);
-            const int j = i + pick_int(w.w[0], L.n_sites - i);
-            const int t = s_order[i];
+    for (int k = tid; k < L.n_sites; k += blockDim.x) {
+        const Philox4 w = philox4x64(A.rep_base + (u64)r, step, 5 + (u64)A.kind, (u64)k, A.seed, 0);
+        s_w0[k] = (unsigned)(w.w[0] >> 32);             // pick_int reads the upper halves
+        s_w1[k] = (unsigned)(w.w[1] >> 32);
+        s_u[k] = unif53(w.w[2]);
+        s_order[k] = (unsigned short)k;
+    }
+    __syncthreads();
+    if (tid == 0)
+        for (int i = 0; i < L.n_sites; ++i) {
+            const int j = i + pick_int((u64)s_w0[i] << 32, L.n_sites - i);
+            const unsigned short t = s_order[i];
             s_order[i] = s_order[j];
             s_order[j] = t;
-            s_li = s_order[i];
-            s_site = L.site[s_li];
-            cur = A.state[s_site];
-            const int k = pick_int(w.w[1], A.site_nstates[s_site] - 1);
-            s_nxt = (k < cur) ? k : k + 1;
-            u = unif53(w.w[2]);
+        }
+    __syncthreads();
+    const float tke = (float)A.tau_ke, kc = (float)A.kc, keo = (float)A.ke_out, kap = (float)A.kappa;
+    for (int i = 0; i < L.n_sites; ++i) {
+        const int li = s_order[i], site = L.site[li];
+        const int a0 = L.first[li], na = L.first[li + 1] - a0;
+        const int cur = A.state[site];
+        const int k1 = pick_int((u64)s_w1[i] << 32, A.site_nstates[site] - 1);
+        const int nxt = (k1 < cur) ? k1 : k1 + 1;
+        const int qo = A.site_q_off[site] + nxt * na;
+        float q_new = 0.0f;
+        if (tid < na) {
+            q_new = A.q_state[qo + tid];
+            const double dq = (double)q_new - (double)s_x[a0 + tid].w;
+            const float h = (float)dq;
+            s_dq[tid] = make_float2(h, (float)(dq - (double)h));
+            s_qnew[tid] = q_new;
         }
         __syncthreads();
-        const int li = s_li, site = s_site, nxt = s_nxt;
-        const int a0 = L.first[li], na = L.first[li + 1] - a0;
-        const int qo = A.site_q_off[site] + nxt * na;
-        for (int a = tid; a < na; a += blockDim.x)
-            s_dq[a] = (double)A.q_state[qo + a] - (double)A.xyzq[base + L.atom[a0 + a]].w;
-        __syncthreads();
         double part = 0.0;
-        for (int t = tid; t < na * na; t += blockDim.x) {
-            const int k = t / na, l = t % na;
-            const int64_t gk = base + L.atom[a0 + k];
-            const float2 Rk = mc_Rh(A, gk);
+        const int pairs = na * na;
+        for (int t = tid; t < pairs; t += blockDim.x) {
+            const int k = t / na, l = t - k * na;
+            const float2 Rk = s_R[a0 + k];
+            const double dk = (double)s_dq[k].x + (double)s_dq[k].y, dl = (double)s_dq[l].x + (double)s_dq[l].y;
             float Akl;
             if (k == l) {
                 Akl = mc_self_term(Rk.x, tke, kc, keo, kap);
-                part += s_dq[k] * s_phi[a0 + k];
+                part += dk * s_phi[a0 + k];
             } else {
-                const int64_t gl = base + L.atom[a0 + l];
-                Akl = mc_pair_term(A.xyzq[gk], Rk, A.xyzq[gl], mc_Rh(A, gl), tke, kc, keo, kap, A.cut2);
+                Akl = mc_pair_term(s_x[a0 + k], Rk, s_x[a0 + l], s_R[a0 + l], tke, kc, keo, kap, A.cut2);
             }
-            part += 0.5 * s_dq[k] * s_dq[l] * (double)Akl;
+            part += 0.5 * dk * dl * (double)Akl;
         }
-        const double dE = block_sum_d(part, sh);
-        if (tid == 0) {
-            const int so = A.site_state_off[site];
-            double dG = dE - (A.G_ref[so + nxt] - A.G_ref[so + cur]);
-            dG += FARADAY * (A.E[r] - A.E0_ref[site]) * (double)(A.n_e[so + nxt] - A.n_e[so + cur]);
-            dG += A.kT * LN10 * (A.pH[r] - A.pKa_ref[site]) * (double)(A.n_H[so + nxt] - A.n_H[so + cur]);
-            const int acc = (dG <= 0.0) || (u < exp(-dG / A.kT));
-            if (A.dG_out) A.dG_out[site] = dG;
-            if (A.acc_out) A.acc_out[site] = (uint8_t)acc;
-            if (acc) A.state[site] = nxt;
-            s_acc = acc;
+        const int busy = min((pairs + 31) >> 5, SWEEP_THREADS / 32);      // warps that hold terms
+        if (wid < busy) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+            if (lane == 0) s_sum[wid] = part;
+        }
+        __syncthreads();
+        if (wid == 0) {
+            double dE = lane < busy ? s_sum[lane] : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dE += __shfl_xor_sync(0xffffffffu, dE, o);
+            if (lane == 0) {
+                const int so = A.site_state_off[site];
+                double dG = dE - (A.G_ref[so + nxt] - A.G_ref[so + cur]);
+                dG += FARADAY * (A.E[r] - A.E0_ref[site]) * (double)(A.n_e[so + nxt] - A.n_e[so + cur]);
+                dG += A.kT * LN10 * (A.pH[r] - A.pKa_ref[site]) * (double)(A.n_H[so + nxt] - A.n_H[so + cur]);
+                const int acc = (dG <= 0.0) || (s_u[i] < exp(-dG / A.kT));
+                if (A.dG_out) A.dG_out[site] = dG;
+                if (A.acc_out) A.acc_out[site] = (uint8_t)acc;
+                if (acc) A.state[site] = nxt;
+                s_acc = acc;
+            }
         }
         __syncthreads();
         if (s_acc) {
-            // rows of every listed atom: phi_m += sum_a dq_a A_ma (charges still old here)
-            for (int m = tid; m < L.n_atoms; m += blockDim.x) {
-                const int64_t gm = base + L.atom[m];
-                const float4 xm = A.xyzq[gm];
-                const float2 Rm = mc_Rh(A, gm);
-                double d = 0.0;
-                for (int a = 0; a < na; ++a) {
-                    const int64_t ga = base + L.atom[a0 + a];
-                    const float Ama = (ga == gm) ? mc_self_term(Rm.x, tke, kc, keo, kap) : mc_pair_term(xm, Rm, A.xyzq[ga], mc_Rh(A, ga), tke, kc, keo, kap, A.cut2);
-                    d += s_dq[a] * (double)Ama;
+            // rows still needed: phi_m += sum_a dq_a A_ma (charges still old here), a warp a site
+            for (int v = i + 1 + wid; v < L.n_sites; v += SWEEP_THREADS / 32) {
+                const int m0 = L.first[s_order[v]], m1 = L.first[s_order[v] + 1];
+                for (int m = m0 + lane; m < m1; m += 32) {
+                    const float4 xm = s_x[m];
+                    const float2 Rm = s_R[m];
+                    Sum2 d;
+                    for (int a = 0; a < na; ++a) {
+                        float Ama;
+                        if (L.atom[a0 + a] == L.atom[m]) {         // an atom of both sites
+                            Ama = mc_self_term(Rm.x, tke, kc, keo, kap);
+                            s_x[m].w = s_qnew[a];
+                        } else {
+                            Ama = mc_pair_term(xm, Rm, s_x[a0 + a], s_R[a0 + a], tke, kc, keo, kap, A.cut2);
+                        }
+                        d.add_product(s_dq[a].x, s_dq[a].y, Ama);
+                    }
+                    s_phi[m] += d.value();
                 }
-                s_phi[m] += d;
             }
             __syncthreads();
-            for (int a = tid; a < na; a += blockDim.x) A.xyzq[base + L.atom[a0 + a]].w = A.q_state[qo + a];
+            if (tid < na) A.xyzq[base + L.atom[a0 + tid]].w = q_new;
         }
         __syncthreads();
     }
@@ -567,7 +660,7 @@ cudaError_t launch_mc_sweep(const MCArgs& a, int32_t M, cudaStream_t s) {
         const cudaError_t e = launch_pdl(k_sweep_rows, dim3((unsigned)a.n_parts, (unsigned)M), dim3(256), 0, s, a);
         if (e != cudaSuccess) return e;
     }
-    return launch_pdl(k_sweep_decide, dim3(M), dim3(256), 0, s, a);
+    return launch_pdl(k_sweep_decide, dim3(M), dim3(SWEEP_THREADS), 0, s, a);
 }
 
 // --- replica exchange (Eq. 14, 15; schedule of Sec. III.B) ----------------------------
