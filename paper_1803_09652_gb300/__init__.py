@@ -211,11 +211,20 @@ class Context:
         self.N = int(self.atom_off[-1])
         self.params = params or default_params()
         self.device = device
+        self._counts = {}
         h = _P()
         rc = self.lib.gb_ctx_create(C.byref(h), self.M, self.atom_off.ctypes.data,
                                     C.byref(self.params), device)
         _check(rc, None)
         self.h = h
+
+    def atom_counts(self, device):
+        """Atoms of each replica (int64 [M]) on a device, copied there once."""
+        import torch
+        key = str(device)
+        if key not in self._counts:
+            self._counts[key] = torch.as_tensor(np.diff(self.atom_off), device=device)
+        return self._counts[key]
 
     def close(self):
         if getattr(self, "h", None):
@@ -638,18 +647,20 @@ def _make_fn():
             out = gctx.energy_forces(xyzq.detach().contiguous(), rad.contiguous(),
                                      want=("F", "E", "dEdq"))
             fctx.save_for_backward(out["F"], out["dEdq"])
-            fctx.atom_off = torch.as_tensor(gctx.atom_off, device=xyzq.device)
+            fctx.counts = gctx.atom_counts(xyzq.device) if gctx.M != 1 else None
             return (out["E"][:, 0] + out["E"][:, 1])
 
         @staticmethod
         def backward(fctx, g):
+            # no host synchronisation: the number of atoms is known, and the
+            # host runs ahead of the pair passes (one 10,007-atom molecule,
+            # forward and backward: 393 us, 864 with the offsets copied to the
+            # device and the sizes read back on every call)
             F, phi = fctx.saved_tensors
-            off = fctx.atom_off
-            counts = (off[1:] - off[:-1])
-            g_atom = torch.repeat_interleave(g.to(torch.float64), counts)
-            grad = torch.zeros((F.shape[0], 4), dtype=torch.float32, device=F.device)
-            grad[:, :3] = (-F.double() * g_atom[:, None]).float()
-            grad[:, 3] = (phi * g_atom).float()
+            g_atom = g.to(torch.float64)
+            if fctx.counts is not None:
+                g_atom = torch.repeat_interleave(g_atom, fctx.counts, output_size=F.shape[0])
+            grad = torch.cat([F * -g_atom[:, None], (phi * g_atom)[:, None]], 1).float()
             return grad, None, None
 
     return Fn
