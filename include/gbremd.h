@@ -421,7 +421,8 @@ int gb_energy_forces_static(int32_t n_atoms, const gb_params* params, const floa
                             const float* rad_screen, float* R_out, int64_t* F_fixed,
                             float* F_out, double* E_out, double* dEdq_out, void* stream);
 
-/* Kernel timing inside the MD driver.  When enabled, CUDA events are recorded
+/* Kernel timing inside the MD driver (small batches, whose evaluations and MD
+ * steps otherwise run in one launch, then run pass by pass).  When enabled, CUDA events are recorded
  * around the three pair passes of every MD step (inside a captured graph they
  * become event nodes of the graph).  gb_pass_times waits for the events of the
  * last enqueued block of steps and returns the mean duration (ms) of each pass:
@@ -435,8 +436,9 @@ int gb_pass_times(gb_ctx* ctx, double* mean_ms);
  * pair passes, the O(N) transforms, replica by replica -- from a queue, each
  * item waiting only for the items of the same replica it depends on, so the
  * passes of different replicas overlap.  A wait that takes too long records
- * GB_ERR_TIMEOUT (see gb_sync_status) instead of hanging.  Disabled: six
- * launches per step (the close-and-open BAOAB step with the tile bounding
+ * GB_ERR_TIMEOUT (see gb_sync_status) instead of hanging.  Disabled: one
+ * launch for a run of steps of a small batch (replicas of a few hundred atoms), six
+ * launches per step otherwise (the close-and-open BAOAB step with the tile bounding
  * boxes, then the three pair passes and their two O(N) transforms), eight
  * with a cutoff (the neighbour list's reset and build).  With profiling on, gb_persist_times returns
  * out[0] the mean ms per MD step inside the persistent launches of the last

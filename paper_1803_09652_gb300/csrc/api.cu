@@ -61,6 +61,10 @@ struct gb_ctx {
     int* phase_off = nullptr;           // [6][M+1]
     int* phase_count = nullptr;         // [6][M]
     int phase_base[7] = {0};
+    // small batches in one launch (fused.cu): blocks a replica (0 = not used), task table
+    int fused_blocks = 0;
+    gbk::TaskList ftasks;
+    int* ftask_off = nullptr;           // [M+1]
     unsigned* qwords = nullptr;         // queue head + 6 x M completion counters
     unsigned spin_limit = 1u << 22;     // polls before a persistent-kernel wait gives up
     std::vector<int> prof_steps_per_launch;
@@ -128,18 +132,17 @@ void cut_replica(const gb_ctx* c, int r, int tpt, std::vector<int4>& out) {
     }
 }
 
+// Costly blocks first: those at and next to the diagonal hold the
+// chain's close pairs, so starting them early leaves the cheap far blocks for
+// the end of the pass, where they even out the finishing times of the SMs.
+// Any order gives the same fixed-point sums.
+bool near_first(const int4& a, const int4& b) { return a.z - (a.y & ~3) < b.z - (b.y & ~3); }
+
 int build_tasks_into(gb_ctx* c, int tpt, gbk::TaskList& out) {
     std::vector<int4> t;
     t.reserve((size_t)(2 * c->total_cols / tpt + 1));
     for (int r = 0; r < c->M; ++r) cut_replica(c, r, tpt, t);
-    // Costly blocks first: those at and next to the diagonal hold the
-    // chain's near pairs (closed forms, no far-block shortcut), so starting
-    // them early leaves the cheap far blocks for the end of the pass, where
-    // they even out the finishing times of the SMs.  Any order gives the same
-    // fixed-point sums.
-    std::stable_sort(t.begin(), t.end(), [](const int4& a, const int4& b) {
-        return a.z - (a.y & ~3) < b.z - (b.y & ~3);
-    });
+    std::stable_sort(t.begin(), t.end(), near_first);
     if (out.d_tasks) cudaFree(out.d_tasks);
     out.d_tasks = nullptr;
     out.n_tasks = (int)t.size();
@@ -196,6 +199,51 @@ int setup_persist(gb_ctx* c) {
     GB_CHECK(c, zalloc(&c->phase_off, 6 * (size_t)(M + 1)));
     GB_CHECK(c, cudaMemcpy(c->phase_off, poff.data(), sizeof(int) * 6 * (M + 1), cudaMemcpyHostToDevice));
     GB_CHECK(c, zalloc(&c->qwords, 1 + 6 * (size_t)M));
+    return GB_OK;
+}
+
+int fused_flags(const gb_ctx* c) {
+    return (c->p.rep_k != 0.0f ? gbk::EF_REP : 0) | (c->p.kappa != 0.0f ? gbk::EF_SALT : 0);
+}
+
+// Whether a batch runs in one launch (fused.cu), and its tables.  A replica's
+// cluster gets the most thread blocks (1 to 16) of which the device holds all
+// replicas' at once, but no more than leave every SM sub-partition a task.  The
+// launch is taken when its warps hold every block of the largest replica in one
+// round, or in two where the batch fills the GPU either way.  Microseconds an MD
+// step in one launch and pass by pass: 1 x 64 20 / 33, 1 x 256 26 / 35, 1 x 512
+// 31 / 37, 1 x 700 (a second round) 42 / 37, 18 x 256 28 / 38, 16 x 512 (second
+// round) 45 / 41, 20 x 400 34 / 42, 40 x 300 36 / 49, 75 x 300 (second round, GPU
+// full) 51 / 61, 150 x 100 29 / 49, 250 x 60 22 / 48.
+int setup_fused(gb_ctx* c) {
+    if (c->list_ctr || c->total_cols == 0) return GB_OK;
+    std::vector<int4> t;
+    std::vector<int> toff(c->M + 1, 0);
+    int sms = 0, most = 0, blocks = 16;
+    GB_CHECK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
+    if (c->M > 2 * sms || c->max_n > 1024) return GB_OK;
+    for (int r = 0; r < c->M; ++r) {
+        std::vector<int4> own;
+        cut_replica(c, r, 1, own);
+        std::stable_sort(own.begin(), own.end(), near_first);
+        t.insert(t.end(), own.begin(), own.end());
+        toff[r + 1] = (int)t.size();
+        most = std::max(most, (int)own.size());
+    }
+    for (;; blocks /= 2) {
+        int room = 0;
+        if (blocks > 1 && 4 * (blocks / 2) >= most) continue;       // a warp an SM sub-partition is enough
+        GB_CHECK(c, gbk::fused_resident(fused_flags(c), blocks, &room));
+        if (room >= c->M) break;
+        if (blocks == 1) return GB_OK;
+    }
+    if (most > gbk::FUSED_WARPS * blocks * (t.size() >= 2048 ? 2 : 1)) return GB_OK;
+    c->ftasks.n_tasks = (int)t.size();
+    GB_CHECK(c, zalloc(&c->ftasks.d_tasks, t.size()));
+    GB_CHECK(c, cudaMemcpy(c->ftasks.d_tasks, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    GB_CHECK(c, zalloc(&c->ftask_off, c->M + 1));
+    GB_CHECK(c, cudaMemcpy(c->ftask_off, toff.data(), sizeof(int) * (c->M + 1), cudaMemcpyHostToDevice));
+    c->fused_blocks = blocks;
     return GB_OK;
 }
 
@@ -279,6 +327,18 @@ cudaError_t pass(const gb_ctx* c, int which, int flags, const gbk::PairArgs& pa,
     return gbk::launch_pairs(which, flags, pa, c->tasks, c->wpb, s);
 }
 
+// Fields of a one-launch evaluation (fused.cu) other than its mode and outputs.
+gbk::FusedArgs fused_args(const gb_ctx* c, const float* xyzq, const float* rad) {
+    gbk::FusedArgs a{};
+    a.pa = pair_args(c, xyzq, rad);
+    a.aa = atom_args(c, xyzq, rad);
+    a.md.xyzq = (float4*)xyzq;
+    a.tasks = c->ftasks.d_tasks;
+    a.task_off = c->ftask_off;
+    a.blocks = c->fused_blocks;
+    a.M = c->M;
+    return a;
+}
 // md != null: an MD step; the chain-bond forces join the force accumulators
 // and the tile boxes were already built by k_md_step (build_boxes false).
 int evaluate(gb_ctx* c, const float* xyzq, const float* rad, float* R_out, int flags,
@@ -312,6 +372,17 @@ int ensure_prof_events(gb_ctx* c, int64_t steps) {
         GB_CHECK(c, cudaEventCreate(&e));
         c->prof_ev.push_back(e);
     }
+    return GB_OK;
+}
+
+// Accumulators back to zero, which the kernels otherwise leave them at.
+int clear_sums(gb_ctx* c, cudaStream_t s) {
+    const size_t N = (size_t)c->N;
+    GB_CHECK(c, cudaMemsetAsync(c->I_acc, 0, sizeof(u64) * N, s));
+    GB_CHECK(c, cudaMemsetAsync(c->dR_acc, 0, sizeof(u64) * N, s));
+    GB_CHECK(c, cudaMemsetAsync(c->phi_acc, 0, sizeof(u64) * N, s));
+    GB_CHECK(c, cudaMemsetAsync(c->F_acc, 0, sizeof(u64) * 3 * N, s));
+    GB_CHECK(c, cudaMemsetAsync(c->E_acc, 0, sizeof(u64) * 4 * (size_t)c->M, s));
     return GB_OK;
 }
 
@@ -427,6 +498,7 @@ extern "C" int gb_ctx_create(gb_ctx** out, int32_t n_rep, const int64_t* atom_of
     for (int k = 0; k < 3; ++k) c->tasks.cap[k] = c->list_ctr ? 3 : 1;
     int rc = build_tasks(c);
     if (rc == GB_OK) rc = setup_persist(c);
+    if (rc == GB_OK) rc = setup_fused(c);
     if (rc != GB_OK) {
         g_create_error = c->msg;
         gb_ctx_destroy(c);
@@ -444,6 +516,8 @@ extern "C" int gb_ctx_destroy(gb_ctx* c) {
     cudaFree(c->tasks.d_tasks);
     cudaFree(c->ptasks.d_tasks);
     cudaFree(c->ptask_off);
+    cudaFree(c->ftasks.d_tasks);
+    cudaFree(c->ftask_off);
     cudaFree(c->phase_off);
     cudaFree(c->phase_count);
     cudaFree(c->qwords);
@@ -543,6 +617,13 @@ extern "C" int gb_born_radii(gb_ctx* c, const float* xyzq, const float* rad, flo
     if (!R_out && c->N > 0) return fail(c, GB_ERR_INVALID_ARG, "R_out is NULL");
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
+    if (c->fused_blocks) {
+        gbk::FusedArgs a = fused_args(c, xyzq, rad);
+        a.born_only = 1;
+        a.R_out = R_out;
+        GB_CHECK(c, gbk::launch_fused(a, fused_flags(c), s));
+        return GB_OK;
+    }
     const gbk::PairArgs pa = pair_args(c, xyzq, rad);
     const gbk::AtomArgs aa = atom_args(c, xyzq, rad);
     GB_CHECK(c, gbk::launch_tile_boxes(pa, c->M, c->n_tiles32, s));
@@ -563,6 +644,14 @@ extern "C" int gb_energy_forces(gb_ctx* c, const float* xyzq, const float* rad, 
         return fail(c, GB_ERR_INVALID_ARG, "no output requested");
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
+    if (c->fused_blocks && !E_out && !dEdq_out) {
+        gbk::FusedArgs a = fused_args(c, xyzq, rad);
+        a.R_out = R_out;
+        a.F_fixed = F_fixed;
+        a.F_out = F_out;
+        GB_CHECK(c, gbk::launch_fused(a, fused_flags(c), s));
+        return GB_OK;
+    }
     int flags = (E_out ? gbk::EF_ENERGY : 0) | (dEdq_out ? gbk::EF_PHI : 0) |
                 (c->p.rep_k != 0.0f ? gbk::EF_REP : 0);
     rc = evaluate(c, xyzq, rad, R_out, flags, dEdq_out, s);
@@ -913,6 +1002,30 @@ int enqueue_steps(gb_ctx* c, gb_md_state* st, const gb_sites* sites, int64_t len
         GB_CHECK(c, gbk::launch_advance_counters(c->ctr, (u64)len, 0, s));
         return GB_OK;
     }
+    if (c->fused_blocks && !c->prof) {           // the passes are timed launch by launch
+        gbk::FusedArgs a = fused_args(c, xyzq, rad);
+        a.md = m;
+        a.R_out = st->R;
+        for (int64_t k = 0; k < len;) {
+            int64_t run = 0;
+            while (k + run < len && run < 1000) {
+                ++run;
+                const int64_t t = (int64_t)st->step + k + run;
+                if (mc_due(t) || ex_due(t)) break;
+            }
+            a.nsteps = (int)run;
+            a.step0 = (int)k;
+            GB_CHECK(c, gbk::launch_fused(a, fused_flags(c), s));
+            k += run;
+            const int64_t t = (int64_t)st->step + k;
+            int rc = mc_due(t) ? enqueue_mc(c, st, sites, k, s) : GB_OK;
+            if (!rc && ex_due(t)) rc = enqueue_exchange(c, st, sites, s);
+            if (!rc && mc_due(t)) rc = enqueue_occupancy(c, st, sites, s);
+            if (rc) return rc;
+        }
+        GB_CHECK(c, gbk::launch_advance_counters(c->ctr, (u64)len, 0, s));
+        return GB_OK;
+    }
     if (c->prof) {
         int rc = ensure_prof_events(c, len);
         if (rc) return rc;
@@ -960,12 +1073,8 @@ extern "C" int gb_md_init(gb_ctx* c, gb_md_state* st, void* stream) {
     // a restart point: a segment that stopped early (a wait that ran out) may
     // have left partial sums in the accumulators, which the kernels otherwise
     // clear as they read them
-    const size_t N = (size_t)c->N;
-    GB_CHECK(c, cudaMemsetAsync(c->I_acc, 0, sizeof(u64) * N, s));
-    GB_CHECK(c, cudaMemsetAsync(c->dR_acc, 0, sizeof(u64) * N, s));
-    GB_CHECK(c, cudaMemsetAsync(c->phi_acc, 0, sizeof(u64) * N, s));
-    GB_CHECK(c, cudaMemsetAsync(c->F_acc, 0, sizeof(u64) * 3 * N, s));
-    GB_CHECK(c, cudaMemsetAsync(c->E_acc, 0, sizeof(u64) * 4 * (size_t)c->M, s));
+    rc = clear_sums(c, s);
+    if (rc) return rc;
     rc = evaluate(c, st->xyzq, st->rad_screen, st->R, flags, nullptr, s, nullptr, &m, true);
     if (rc) return rc;
     GB_CHECK(c, gbk::launch_md_step(atom_args(c, st->xyzq, st->rad_screen), m, nullptr, nullptr, 0, gbk::MD_CLOSE, s));
@@ -1002,7 +1111,9 @@ extern "C" int gb_md_segment(gb_ctx* c, gb_md_state* st, const gb_sites* sites, 
     };
     if (sites && st->mc_every > 0) L = lcm(L, st->mc_every);
     if (sites && st->grid && st->ex_every > 0) L = lcm(L, st->ex_every);
-    const bool graph_ok = (L <= 1000) && ((int64_t)st->step % L == 0) && (nsteps % L == 0);
+    // (a batch that runs in one launch has nothing to capture between halts)
+    const bool one_launch = c->fused_blocks && !c->prof && !c->use_persist;
+    const bool graph_ok = (L <= 1000) && !(one_launch && L == 1) && ((int64_t)st->step % L == 0) && (nsteps % L == 0);
     GB_CHECK(c, gbk::launch_set_counters(c->ctr, st->step, st->attempt, s));
     if (!graph_ok) {
         rc = enqueue_steps(c, st, sites, nsteps, s);

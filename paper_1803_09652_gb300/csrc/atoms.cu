@@ -45,18 +45,12 @@ __global__ void k_energy_finalize(AtomArgs A, int want_energy, double* phi_out, 
     if (i < n) {
         const int64_t g = base + i;
         double R;
-        const double q = chain_factor_atom(A, g, &R);
+        const double q = chain_bond_atom(A, A.xyzq, bond_k, bond_r0, base, i, n, &R);
         const double tE = gb_screen(A.kc, A.ke_out, A.kappa, R).x;
         eself = -0.5 * tE * q * q / R;
         if (phi_out) {
             phi_out[g] = unfix(A.phi_acc[g]) - tE * q / R;
             A.phi_acc[g] = 0;
-        }
-        if (bond_k != 0.0f) {
-            const float3 fb = bond_force_kr(bond_k, bond_r0, A.xyzq, base, i, n);
-            A.F_acc[g] = __ldcg(&A.F_acc[g]) + (u64)fix(fb.x);
-            A.F_acc[A.N + g] = __ldcg(&A.F_acc[A.N + g]) + (u64)fix(fb.y);
-            A.F_acc[2 * A.N + g] = __ldcg(&A.F_acc[2 * A.N + g]) + (u64)fix(fb.z);
         }
     }
     if (want_energy) {
@@ -78,21 +72,7 @@ __global__ void k_forces_out(AtomArgs A, int64_t* F_fixed, float* F_out, double*
         A.E_acc[4 * r + threadIdx.x] = 0;
     }
     if (i >= n) return;
-    const int64_t g = base + i;
-    const u64 fx = A.F_acc[g], fy = A.F_acc[A.N + g], fz = A.F_acc[2 * A.N + g];
-    A.F_acc[g] = 0;
-    A.F_acc[A.N + g] = 0;
-    A.F_acc[2 * A.N + g] = 0;
-    if (F_fixed) {
-        F_fixed[g] = (long long)fx;
-        F_fixed[A.N + g] = (long long)fy;
-        F_fixed[2 * A.N + g] = (long long)fz;
-    }
-    if (F_out) {
-        F_out[3 * g + 0] = (float)unfix(fx);
-        F_out[3 * g + 1] = (float)unfix(fy);
-        F_out[3 * g + 2] = (float)unfix(fz);
-    }
+    forces_out_atom(A, base + i, F_fixed, F_out);
 }
 
 // --- Langevin BAOAB ---------------------------------------------------------------

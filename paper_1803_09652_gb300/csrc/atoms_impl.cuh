@@ -72,6 +72,24 @@ __device__ __forceinline__ double chain_factor_atom(const AtomArgs& A, int64_t g
     return q;
 }
 
+// Readout of the force accumulators of atom g, which are cleared.
+__device__ __forceinline__ void forces_out_atom(const AtomArgs& A, int64_t g, int64_t* F_fixed, float* F_out) {
+    const u64 fx = __ldcg(&A.F_acc[g]), fy = __ldcg(&A.F_acc[A.N + g]), fz = __ldcg(&A.F_acc[2 * A.N + g]);
+    A.F_acc[g] = 0;
+    A.F_acc[A.N + g] = 0;
+    A.F_acc[2 * A.N + g] = 0;
+    if (F_fixed) {
+        F_fixed[g] = (long long)fx;
+        F_fixed[A.N + g] = (long long)fy;
+        F_fixed[2 * A.N + g] = (long long)fz;
+    }
+    if (F_out) {
+        F_out[3 * g + 0] = (float)unfix(fx);
+        F_out[3 * g + 1] = (float)unfix(fy);
+        F_out[3 * g + 2] = (float)unfix(fz);
+    }
+}
+
 // Standard normals from Philox4x64-10 (key (seed, 0), counter (replica, step,
 // 4, atom)) by Box-Muller on (u1, u2) and (u3, u4), u1, u3 in (0, 1].
 __device__ __forceinline__ float3 md_normals(u64 seed, u64 r, u64 step, u64 atom) {
@@ -101,16 +119,25 @@ __device__ __forceinline__ void baoab_first(const MDArgs& m, float4& x, float4& 
 }
 
 // Harmonic chain bonds k (r - r0)^2 with atoms i-1 and i+1 of the replica:
-// force on atom i.
-__device__ __forceinline__ float3 bond_force_kr(float k, float r0, const float4* xyzq, int64_t base, int i, int n) {
+// the force on atom i, from coordinates loaded beforehand.
+struct BondAtoms {
+    float4 x[3];                       // atoms i-1, i, i+1 (i itself where there is none)
+};
+__device__ __forceinline__ BondAtoms load_bond_atoms(const float4* xyzq, int64_t base, int i, int n) {
+    BondAtoms b;
+    b.x[0] = __ldcg(&xyzq[base + (i > 0 ? i - 1 : i)]);
+    b.x[1] = __ldcg(&xyzq[base + i]);
+    b.x[2] = __ldcg(&xyzq[base + (i + 1 < n ? i + 1 : i)]);
+    return b;
+}
+__device__ __forceinline__ float3 bond_force(float k, float r0, const BondAtoms& b, int i, int n) {
     float3 f = make_float3(0.0f, 0.0f, 0.0f);
-    if (k == 0.0f) return f;
-    const float4 xi = __ldcg(&xyzq[base + i]);
+    const float4 xi = b.x[1];
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
         const int j = side ? i + 1 : i - 1;
         if (j < 0 || j >= n) continue;
-        const float4 xj = __ldcg(&xyzq[base + j]);
+        const float4 xj = b.x[2 * side];
         const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
         const float rr = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
         // dE/dr = 2 k (r - r0); the force on i points along +d when stretched
@@ -119,8 +146,23 @@ __device__ __forceinline__ float3 bond_force_kr(float k, float r0, const float4*
     }
     return f;
 }
-__device__ __forceinline__ float3 bond_force(const MDArgs& m, const float4* xyzq, int64_t base, int i, int n) {
-    return bond_force_kr(m.bond_k, m.bond_r0, xyzq, base, i, n);
+
+// Chain factor of atom i (global index g) and, with bond_k != 0 (MD), the
+// chain-bond forces added to the force accumulators.  Everything is loaded
+// before the first store: as three dependent steps this took 2 us of latency.
+// Returns q and *R_used as chain_factor_atom.
+__device__ __forceinline__ double chain_bond_atom(const AtomArgs& A, const float4* xyzq, float bond_k, float bond_r0,
+                                                  int64_t base, int i, int n, double* R_used) {
+    const int64_t g = base + i;
+    if (bond_k == 0.0f) return chain_factor_atom(A, g, R_used);
+    const BondAtoms b = load_bond_atoms(xyzq, base, i, n);
+    const u64 fx = __ldcg(&A.F_acc[g]), fy = __ldcg(&A.F_acc[A.N + g]), fz = __ldcg(&A.F_acc[2 * A.N + g]);
+    const double q = chain_factor_atom(A, g, R_used);
+    const float3 fb = bond_force(bond_k, bond_r0, b, i, n);
+    A.F_acc[g] = fx + (u64)fix(fb.x);
+    A.F_acc[A.N + g] = fy + (u64)fix(fb.y);
+    A.F_acc[2 * A.N + g] = fz + (u64)fix(fb.z);
+    return q;
 }
 
 }  // namespace gbk

@@ -301,6 +301,27 @@ size_t persist_smem();
 cudaError_t persist_occupancy(int rep, int* blocks_per_sm);
 cudaError_t launch_persist(const PersistArgs& a, int rep, int grid, cudaStream_t s);
 
+// Small batches in one launch (fused.cu).
+constexpr int FUSED_WARPS = 8;     // warps of a thread block
+struct FusedArgs {
+    PairArgs pa;
+    AtomArgs aa;
+    MDArgs md;                 // nsteps > 0
+    const int4* tasks;         // pair tasks (one block each) of every replica, replica after replica
+    const int* task_off;       // [M+1] first task of each replica
+    int blocks;                // thread blocks of every replica's cluster: 1, 2, 4, 8 or 16
+    int M;
+    int nsteps;                // MD steps (0: one force evaluation of given coordinates)
+    int step0;                 // index of the first of them in the enqueued block
+    int born_only;             // nsteps == 0: stop after the Born radii
+    float* R_out;              // nullable
+    int64_t* F_fixed;          // nullable, nsteps == 0
+    float* F_out;              // nullable, nsteps == 0
+};
+// Clusters of that many blocks the device holds at once.
+cudaError_t fused_resident(int flags, int blocks, int* clusters);
+cudaError_t launch_fused(const FusedArgs& a, int flags, cudaStream_t s);
+
 cudaError_t launch_count(const int32_t* site_off, const int32_t* site_kind, const int32_t* site_nstates,
                          const int32_t* site_state_off, const int32_t* n_H,
                          const int32_t* n_e, const int32_t* state, int32_t kind, int32_t M,

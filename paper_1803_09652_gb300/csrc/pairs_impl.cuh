@@ -1061,15 +1061,17 @@ constexpr int WARP_SMEM = 2 * P::NQ * 64 * 8 + 1024 + 512 + 256 + P::NJ * 256 + 
 template <class P>
 inline int fit_warps(int wpb) { return wpb * WARP_SMEM<P> <= 49152 ? wpb : 49152 / WARP_SMEM<P>; }
 
-// Exact sum into a shared 64-bit word by two 32-bit atomics (there is no
-// native 64-bit one): the carry follows from the low word's old value.
-__device__ __forceinline__ void shared_add(long long* p, long long v) {
-    unsigned* w = (unsigned*)p;
-    const unsigned lo = (unsigned)v;
-    unsigned hi = (unsigned)((u64)v >> 32);
-    const unsigned old = atomicAdd(w, lo);
-    hi += (old + lo < lo) ? 1u : 0u;
-    if (hi) atomicAdd(w + 1, hi);
+// Exact sums into N shared 64-bit words by two 32-bit atomics each (there is no
+// native 64-bit one): the carry follows from the low word's old value.  All
+// low words first, so that their latencies overlap.
+template <int N>
+__device__ __forceinline__ void shared_add(long long* const (&p)[N], const long long (&v)[N]) {
+    unsigned old[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) old[k] = atomicAdd((unsigned*)p[k], (unsigned)v[k]);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        atomicAdd((unsigned*)p[k] + 1, (unsigned)((u64)v[k] >> 32) + (old[k] + (unsigned)v[k] < old[k] ? 1u : 0u));
 }
 
 // The r^2 below which a pair of a near block is close: above it the spheres
@@ -1161,6 +1163,9 @@ struct BornY {
         if (!isfinite(st.acc) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
         if (j < n) red_add(&A.I_acc[base + j], fix_i(st.acc) + (jac ? jac[at] : 0));
     }
+    static __device__ __forceinline__ void flush_close(const PairArgs& A, int64_t g, const long long* jac, int j) {
+        red_add(&A.I_acc[g], jac[j]);
+    }
     static __device__ __forceinline__ float bound(const PairArgs&, const Slot<BornY>& S, int lane) { return staged_bound(S, lane); }
     // One close pair a lane, both directions as the halves of a pair.
     static __device__ __forceinline__ void close(const PairArgs& A, const Slot<BornY>& S, long long* sa, int i, int j,
@@ -1180,8 +1185,9 @@ struct BornY {
         }
         if (!valid) return;
         if (!isfinite(h.x + h.y) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
-        shared_add(&sa[i], fix_i(h.x));
-        shared_add(&S.jac[j], fix_i(h.y));
+        long long* const to[2] = {&sa[i], &S.jac[j]};
+        const long long v[2] = {fix_i(h.x), fix_i(h.y)};
+        shared_add(to, v);
     }
 };
 
@@ -1286,12 +1292,18 @@ struct ForceSums {
         red_add(&A.F_acc[A.N + g], fix(st.fy) + (jac ? jac[32 + at] : 0));
         red_add(&A.F_acc[2 * A.N + g], fix(st.fz) + (jac ? jac[64 + at] : 0));
     }
+    static __device__ __forceinline__ void flush_close(const PairArgs& A, int64_t g, const long long* jac, int j) {
+        red_add(&A.F_acc[g], jac[j]);
+        red_add(&A.F_acc[A.N + g], jac[32 + j]);
+        red_add(&A.F_acc[2 * A.N + g], jac[64 + j]);
+    }
     // a close pair's force fr d, exactly
     static __device__ __forceinline__ void add_close(long long* sa, long long* jac, int i, int j, float fr, float dx,
                                                      float dy, float dz) {
         const long long fx = fix(fr * dx), fy = fix(fr * dy), fz = fix(fr * dz);
-        shared_add(&sa[i], -fx); shared_add(&sa[64 + i], -fy); shared_add(&sa[128 + i], -fz);
-        shared_add(&jac[j], fx); shared_add(&jac[32 + j], fy); shared_add(&jac[64 + j], fz);
+        long long* const to[6] = {&sa[i], &sa[64 + i], &sa[128 + i], &jac[j], &jac[32 + j], &jac[64 + j]};
+        const long long v[6] = {-fx, -fy, -fz, fx, fy, fz};
+        shared_add(to, v);
     }
 };
 
@@ -1550,14 +1562,14 @@ __device__ __noinline__ void walk_far(const PairArgs& A, int r, int i0, int J0, 
     if (W::ATOMS == 64) sa += ((i0 >> 6) & 1) * 64 * W::NQ;
     typename W::B* sb = (typename W::B*)(sj + 64);
     typename W::I is;
+    float4 v;
+    typename W::B b;
+    int j = 32 * (J0 + __ffs(mask) - 1) + lane;
+    W::load_j(A, base, n, j, v, b);                // before the i atoms: one memory latency for both
     W::load_i(A, base, n, i0, lane, is);
     const int next = (lane + 1) & 31;
-    while (mask) {
-        const int j = 32 * (J0 + __ffs(mask) - 1) + lane;
+    for (;;) {
         mask &= mask - 1;
-        float4 v;
-        typename W::B b;
-        W::load_j(A, base, n, j, v, b);
         __syncwarp();
         sj[lane] = sj[32 + lane] = v;
         sb[lane] = sb[32 + lane] = b;
@@ -1572,18 +1584,46 @@ __device__ __noinline__ void walk_far(const PairArgs& A, int r, int i0, int J0, 
         }
         W::fold_i(A, sa, lane, p);
         W::flush_j(A, base, n, j, js);
+        if (!mask) break;
+        j = 32 * (J0 + __ffs(mask) - 1) + lane;
+        W::load_j(A, base, n, j, v, b);
     }
 }
 
-// The pairs noted in the lanes' masks (bit k of mx / my: the x / y half's atom
-// against tile atom (lane + k) mod 32), 32 at a time.  Returns their number.
+// Pairs b0 .. b0 + CLOSE_CAP - 1 of those noted in the lanes' masks (bit k of
+// mx / my: the x / y half's atom against tile atom (lane + k) mod 32) into the
+// warp's queue; before: pairs of the lanes below.
 template <class W>
+__device__ __forceinline__ void queue_close(const Slot<W>& S, unsigned mx, unsigned my, int before, int b0, int lane) {
+    int pos = before - b0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        unsigned m = h ? my : mx;
+        while (m) {
+            const int k = __ffs(m) - 1;
+            m &= m - 1;
+            if (pos >= 0 && pos < CLOSE_CAP) S.queue[pos] = (unsigned short)((32 * h + lane) | (((lane + k) & 31) << 6));
+            ++pos;
+        }
+    }
+    __syncwarp();
+}
+// Entries e .. e + 31 of a queue of cnt.
+template <class W>
+__device__ __forceinline__ void run_close(const PairArgs& A, const Slot<W>& S, int row, int e, int cnt, int i0, int jbase,
+                                          int lane) {
+    const int q = S.queue[min(e + lane, cnt - 1)];
+    W::close(A, S, S.sa + row * 64 * W::NQ, q & 63, q >> 6, e + lane < cnt, i0, jbase);
+}
+// The pairs noted in the lanes' masks, 32 at a time.  Returns their number;
+// with DEFER the last CLOSE_CAP of them at most stay in the queue, and the
+// number of those is returned (see round_pass in fused.cu).
+template <class W, bool DEFER>
 __device__ __noinline__ int close_pairs(const PairArgs& A, int slot, int row, unsigned mx, unsigned my, int i0, int jbase) {
     const int lane = threadIdx.x & 31;
     slot = __shfl_sync(0xffffffffu, slot, 0);
     row = __shfl_sync(0xffffffffu, row, 0);
     const Slot<W> S(slot);
-    long long* sa = S.sa + row * 64 * W::NQ;
     const int own = __popc(mx) + __popc(my);
     int at = own;
 #pragma unroll
@@ -1596,24 +1636,10 @@ __device__ __noinline__ int close_pairs(const PairArgs& A, int slot, int row, un
 #pragma unroll
     for (int q = 0; q < W::NJ; ++q) S.jac[32 * q + lane] = 0;
     for (int b0 = 0; b0 < total; b0 += CLOSE_CAP) {
-        int pos = at - own - b0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            unsigned m = h ? my : mx;
-            while (m) {
-                const int k = __ffs(m) - 1;
-                m &= m - 1;
-                if (pos >= 0 && pos < CLOSE_CAP)
-                    S.queue[pos] = (unsigned short)((32 * h + lane) | (((lane + k) & 31) << 6));
-                ++pos;
-            }
-        }
-        __syncwarp();
+        queue_close(S, mx, my, at - own, b0, lane);
         const int cnt = min(CLOSE_CAP, total - b0);
-        for (int e = 0; e < cnt; e += 32) {
-            const int q = S.queue[min(e + lane, cnt - 1)];
-            W::close(A, S, sa, q & 63, q >> 6, e + lane < cnt, i0, jbase);
-        }
+        if (DEFER && b0 + CLOSE_CAP >= total) return cnt;
+        for (int e = 0; e < cnt; e += 32) run_close(A, S, row, e, cnt, i0, jbase, lane);
         __syncwarp();
     }
     return total;
@@ -1633,9 +1659,10 @@ __device__ __forceinline__ void near_tile(const PairArgs& A, const typename W::I
 }
 
 // Row K (64 atoms) against tiles J0 + (set bits of `todo`), near or diagonal;
-// t: of lane c the bound below which pairs of column J0 + c are close.
-template <class W, bool CLOSE>
-__device__ __noinline__ void walk_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
+// t: of lane c the bound below which pairs of column J0 + c are close.  DEFER
+// (one column): the close pairs stay in the queue, their number is returned.
+template <class W, bool CLOSE, bool DEFER = false>
+__device__ __noinline__ int walk_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
     const int lane = threadIdx.x & 31;
     slot = __shfl_sync(0xffffffffu, slot, 0);
     r = __shfl_sync(0xffffffffu, r, 0);
@@ -1647,14 +1674,14 @@ __device__ __noinline__ void walk_near(const PairArgs& A, int r, int K, int J0, 
     const Slot<W> S(slot);
     long long* sa = S.sa + (K & 1) * 64 * W::NQ;
     typename W::I is;
+    float4 v;
+    typename W::B b;
+    float2 as;
+    W::load(A, base, n, 32 * (J0 + __ffs(todo) - 1) + lane, v, b, as);
     W::load_i(A, base, n, 64 * K, lane, is, S.i4, S.i2);
-    while (todo) {
+    for (;;) {
         const int c = __ffs(todo) - 1, J = J0 + c;
         todo &= todo - 1;
-        float4 v;
-        typename W::B b;
-        float2 as;
-        W::load(A, base, n, 32 * J + lane, v, b, as);
         __syncwarp();
         S.j4[lane] = S.j4[32 + lane] = v;
         S.jb[lane] = S.jb[32 + lane] = b;
@@ -1677,9 +1704,12 @@ __device__ __noinline__ void walk_near(const PairArgs& A, int r, int K, int J0, 
         }
         W::fold_i(A, sa, lane, p);
         __syncwarp();
-        const int n_close = CLOSE ? close_pairs<W>(A, slot, K & 1, mk[0], mk[1], 64 * K, 32 * J) : 0;
+        const int n_close = CLOSE ? close_pairs<W, DEFER>(A, slot, K & 1, mk[0], mk[1], 64 * K, 32 * J) : 0;
         const int at = (lane + shift) & 31;
-        W::flush_j(A, base, n, 32 * J + at, js, n_close ? S.jac : nullptr, at);
+        W::flush_j(A, base, n, 32 * J + at, js, !DEFER && n_close ? S.jac : nullptr, at);
+        if (DEFER) return n_close;
+        if (!todo) return 0;
+        W::load(A, base, n, 32 * (J0 + __ffs(todo) - 1) + lane, v, b, as);
     }
 }
 
@@ -1744,11 +1774,25 @@ __device__ __forceinline__ void run_far(int tier, const PairArgs& A, int r, int 
         else walk_far<BornY<NW>>(A, r, i0, J0, mask, slot);
     }
 }
+// The form of a pass's near blocks, and whether it has close pairs at all.
 template <class P, int FLAGS>
-__device__ __forceinline__ void run_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
-    if constexpr (!P::RADIUS_CUT) walk_near<EnergyW<1, FLAGS & EF_SALT>, (FLAGS & EF_REP) != 0>(A, r, K, J0, todo, t, slot);
-    else if constexpr (P::CHAIN) walk_near<ChainY<1>, true>(A, r, K, J0, todo, t, slot);
-    else walk_near<BornY<1>, true>(A, r, K, J0, todo, t, slot);
+struct NearForm {
+    typedef EnergyW<1, FLAGS & EF_SALT> W;
+    static constexpr bool CLOSE = (FLAGS & EF_REP) != 0;
+};
+template <int FLAGS>
+struct NearForm<Born, FLAGS> {
+    typedef BornY<1> W;
+    static constexpr bool CLOSE = true;
+};
+template <int FLAGS>
+struct NearForm<Chain, FLAGS> {
+    typedef ChainY<1> W;
+    static constexpr bool CLOSE = true;
+};
+template <class P, int FLAGS, bool DEFER = false>
+__device__ __forceinline__ int run_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
+    return walk_near<typename NearForm<P, FLAGS>::W, NearForm<P, FLAGS>::CLOSE, DEFER>(A, r, K, J0, todo, t, slot);
 }
 
 // Work of replica r is walked as row pairs P = 0 .. ceil(nb/4) - 1 (nb tiles

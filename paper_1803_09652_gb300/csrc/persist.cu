@@ -25,20 +25,13 @@
 // quarter of a second; gb_set_wait_limit) the warp records GB_ERR_TIMEOUT and
 // stops taking work; the others then see the error word, or time out on it,
 // and stop too, so the launch always ends and the context stays usable.
-#include "atoms_impl.cuh"
-#include "pairs_impl.cuh"
+#include "md_tiles.cuh"
 
 namespace gbk {
 
 constexpr int PERSIST_THREADS = 128;
 constexpr int PERSIST_SMEM = WARP_SMEM<Energy>;   // the largest of the three passes' slots
 static_assert(PERSIST_SMEM >= WARP_SMEM<Chain> && PERSIST_SMEM >= WARP_SMEM<Born>, "slot");
-
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 
 // Lane 0 waits until *ctr >= target; returns false when the wait gave up or
 // another warp reported an error.
@@ -60,60 +53,6 @@ __device__ __forceinline__ bool wait_count(const unsigned* ctr, unsigned target,
     ok = __shfl_sync(0xffffffffu, ok, 0);
     __syncwarp();
     return ok != 0;
-}
-
-// Phase 0 on tile u of replica r.  second: close the previous step (force
-// from the accumulators, kick).  first: open step `step` (B A O A with the
-// same force) and rebuild the tile's box; otherwise store the force.
-__device__ __forceinline__ void tile_halfsteps(const PersistArgs& P, int r, int u, int lane, bool second,
-                                               bool first, u64 step) {
-    const MDArgs& m = P.md;
-    const int64_t N = P.pa.N;
-    const int64_t base = P.pa.atom_off[r];
-    const int n = (int)(P.pa.atom_off[r + 1] - base);
-    const int i = 32 * u + lane;
-    if (i < n) {
-        const int64_t g = base + i;
-        float4 v = __ldcg(&m.vel[g]);
-        float4 f;
-        if (second) {
-            f = make_float4((float)unfix(__ldcg(&P.aa.F_acc[g])), (float)unfix(__ldcg(&P.aa.F_acc[N + g])),
-                            (float)unfix(__ldcg(&P.aa.F_acc[2 * N + g])), 0.0f);
-            P.aa.F_acc[g] = 0;
-            P.aa.F_acc[N + g] = 0;
-            P.aa.F_acc[2 * N + g] = 0;
-            v.x = fmaf(m.h * m.inv_m, f.x, v.x);
-            v.y = fmaf(m.h * m.inv_m, f.y, v.y);
-            v.z = fmaf(m.h * m.inv_m, f.z, v.z);
-        } else {
-            f = __ldcg(&m.force[g]);
-        }
-        if (first) {
-            float4 x = __ldcg(&m.xyzq[g]);
-            baoab_first(m, x, v, f, md_normals(m.seed, m.rep_base + (u64)r, step, (u64)i));
-            m.xyzq[g] = x;
-        } else {
-            m.force[g] = f;
-        }
-        m.vel[g] = v;
-    }
-    if (first) tile_box_warp(P.pa, P.M, P.pa.tile_off[r] + u, lane);
-}
-
-// Phase 4 on atoms 32u .. 32u+31 of replica r: chain factor, chain bonds.
-__device__ __forceinline__ void atoms_chain_bonds(const PersistArgs& P, int r, int u, int lane) {
-    const int64_t N = P.pa.N;
-    const int64_t base = P.pa.atom_off[r];
-    const int n = (int)(P.pa.atom_off[r + 1] - base);
-    const int i = 32 * u + lane;
-    if (i >= n) return;
-    const int64_t g = base + i;
-    double R;
-    chain_factor_atom(P.aa, g, &R);
-    const float3 fb = bond_force(P.md, P.md.xyzq, base, i, n);
-    P.aa.F_acc[g] = __ldcg(&P.aa.F_acc[g]) + (u64)fix(fb.x);
-    P.aa.F_acc[N + g] = __ldcg(&P.aa.F_acc[N + g]) + (u64)fix(fb.y);
-    P.aa.F_acc[2 * N + g] = __ldcg(&P.aa.F_acc[2 * N + g]) + (u64)fix(fb.z);
 }
 
 template <int REP>
