@@ -54,7 +54,7 @@ struct TaskList {
     int n_tasks = 0;
     bool small = false;        // every replica has at most SMALL_TILES tiles
     // register cap of each pass's kernel (Born, energy, chain), as 256-thread
-    // blocks per SM: 1 (compiler's choice), 3 (80 registers) or 4 (64)
+    // blocks per SM: 1 (at most 128 registers), 3 (80) or 4 (64)
     int cap[3] = {1, 1, 1};
 };
 

@@ -15,10 +15,9 @@
 //
 // Pass 1 (Born integrals), pass 2 (GB + Coulomb energy, direct forces, dE/dR,
 // optional dE/dq and soft repulsion) and pass 3 (Born-radius chain rule)
-// share the walk (walk_task).  The general pair code of each pass (Born,
-// Energy, Chain) serves blocks that straddle a cutoff and evaluations that
-// want energies or dE/dq; every other block runs one of the forms under
-// "blocks by distance".
+// share the walk (walk_task).  Blocks run one of the forms under "blocks by
+// distance"; the general code of pass 2 (Energy) serves blocks that straddle
+// the pair cutoff and evaluations that want energies or dE/dq.
 #pragma once
 
 #include "common.cuh"
@@ -31,14 +30,6 @@ namespace gbk {
 // -(dH/dr)/r = 1/2 s^3 r^-6 h(x^2), with g, h the fitted polynomials: no
 // cancellation and no MUFU.
 __device__ __forceinline__ bool far_ok(float r, float lim, float y) { return (r >= lim) && (y <= GB_POLY_YMAX); }
-
-// True (warp-uniform) when every pair of this warp step has y <= GB_POLY_YFAR,
-// where the lower-degree far-field polynomials reach the same FP32 accuracy.
-// The chain's tiles are spatially compact, so most steps qualify.
-__device__ __forceinline__ bool all_far(float2 a, float2 b) {
-    const float m = fmaxf(fmaxf(a.x, a.y), fmaxf(b.x, b.y));
-    return __all_sync(0xffffffffu, m <= GB_POLY_YFAR);
-}
 
 // --- packed FP32x2 helpers ----------------------------------------------------------
 typedef float2 f2;
@@ -156,25 +147,49 @@ __device__ __forceinline__ f2 hct_closed_fr2(f2 r, f2 rinv, f2 a, f2 s) {
     return make_float2(a.x >= U.x ? 0.0f : fr.x, a.y >= U.y ? 0.0f : fr.y);
 }
 
+// J(z) = int_0^z t^2/(1-t) dt = -ln(1 - z) - z - z^2/2 = z^3 q(z): the fitted series
+// of positive terms of poly_coeffs.h (gb_poly_q for z <= 1/2, gb_poly_q_hi for
+// z <= 3/4), and beyond that the logarithm (UL = 1 / (1 - z)), where its terms
+// cancel by less than a factor 10; each range behind a warp vote over the lanes
+// that use the result.
+__device__ __forceinline__ f2 shell_J(f2 z, f2 UL, bool use0, bool use1) {
+    const f2 z2 = mul2(z, z), z3 = mul2(z2, z);
+    f2 J = mul2(z3, gb_poly_q2(z));
+    if (__any_sync(0xffffffffu, (use0 && z.x > GB_POLY_ZJ) || (use1 && z.y > GB_POLY_ZJ))) {
+        const f2 Jh = mul2(z3, gb_poly_q_hi2(add2(z, F2(-GB_POLY_ZMID))));
+        J = make_float2(z.x > GB_POLY_ZJ ? Jh.x : J.x, z.y > GB_POLY_ZJ ? Jh.y : J.y);
+        if (__any_sync(0xffffffffu, (use0 && z.x > GB_POLY_ZJ2) || (use1 && z.y > GB_POLY_ZJ2))) {
+            const f2 Jl = add2(logv(UL), neg2(fma2(F2(0.5f), z2, z)));
+            J = make_float2(z.x > GB_POLY_ZJ2 ? Jl.x : J.x, z.y > GB_POLY_ZJ2 ? Jl.y : J.y);
+        }
+    }
+    return J;
+}
+
 // --- the same integral restricted to the ball |y - x_i| < rc (Born-radius cutoff) ---
 // Shells about x_i now run from L to U' = min(U, rc): the bracket of
 // hct_closed2 with U' in place of U when L < U' (else no shell term), and the
 // engulfed part 2 (1/a - 1/min(L, rc)) when a < s - r and a < rc.  irc = 1/rc.
-// Serves the pairs of blocks that straddle the cutoff, where sphere j reaches
-// past rc (r + s > rc); it is exact (to rounding) for every geometry, so the
-// lanes of such a step that do not reach past rc may take it too.
+// With z = (U' - L) / U' the bracket is
+//   { z [s^2 - (r - L)^2] / L^2 + z^2 [r^2 - L^2 - s^2] / (2 L^2) - J(z) } / (2r),
+// whose terms do not cancel as 1/L - 1/U' and the logarithm do: a pair's error
+// is 1.2e-7 rms of the mean integral of overlapping pairs against 3.3e-7, and
+// with rgbmax = 2.6 A, where nearly every bonded pair is cut, that decides R.
+// It is exact (to rounding) for every geometry: any pair may take it.
 __device__ __forceinline__ f2 hct_cut2(f2 r, f2 rinv, f2 a, f2 s, float rc, float irc) {
     const f2 U = add2(r, s);
     const f2 Up = make_float2(fminf(U.x, rc), fminf(U.y, rc));
     const f2 rs = add2(r, neg2(s));
     const f2 L = make_float2(fmaxf(a.x, fabsf(rs.x)), fmaxf(a.y, fabsf(rs.y)));
-    const f2 iU = rcp2(Up), iL = rcp2(L);
-    const f2 dU2 = add2(mul2(iU, iU), neg2(mul2(iL, iL)));
-    const f2 w = fma2(neg2(mul2(s, s)), rinv, r);
-    f2 b = fma2(mul2(F2(0.25f), w), dU2, add2(iL, neg2(iU)));
-    b = fma2(mul2(F2(0.5f), rinv), logv(mul2(L, iU)), b);
-    b.x = (L.x < Up.x) ? b.x : 0.0f;
-    b.y = (L.y < Up.y) ? b.y : 0.0f;
+    const bool in0 = L.x < Up.x, in1 = L.y < Up.y;
+    const f2 iU = rcp2(Up), iL = rcp2(L), iL2 = mul2(iL, iL);
+    const f2 z = mul2(add2(Up, neg2(L)), iU), J = shell_J(z, mul2(Up, iL), in0, in1);
+    const f2 d = add2(r, neg2(L));
+    const f2 c1 = mul2(mul2(add2(s, neg2(d)), add2(s, d)), iL2);
+    const f2 c2 = mul2(fma2(d, add2(r, L), neg2(mul2(s, s))), iL2);
+    f2 b = mul2(mul2(F2(0.5f), rinv), fma2(z, fma2(mul2(F2(0.5f), z), c2, c1), neg2(J)));
+    b.x = in0 ? b.x : 0.0f;
+    b.y = in1 ? b.y : 0.0f;
     const f2 iLc = make_float2(L.x < rc ? iL.x : irc, L.y < rc ? iL.y : irc);
     const f2 eng = mul2(F2(2.0f), add2(rcp2(a), neg2(iLc)));
     b.x += (a.x < -rs.x && a.x < rc) ? eng.x : 0.0f;
@@ -220,15 +235,10 @@ static __device__ __noinline__ f2 hct_cut_fr2(f2 r, f2 rinv, f2 a, f2 s, float r
 // Disjoint spheres (r >= a + s) reaching past rc: the shells run from
 // L = r - s to U' = min(r + s, rc), and with w = U' - L, z = w / U' the
 // integral takes a form without cancelling O(1/L) terms,
-//   H = 1/(4r) [ (s/L) z^2 - J(z) ],   J(z) = -ln(1 - z) - z - z^2/2 = z^3 q(z)
-// (J = int_0^z t^2/(1-t) dt; q the fitted series of positive terms of
-// poly_coeffs.h: gb_poly_q for z <= 1/2, gb_poly_q_hi for z <= 3/4, which
-// covers every pair of disjoint spheres of the usual radius sets, and beyond
-// that J from the logarithm, where its terms cancel by less than a factor 10;
-// each range behind a warp vote over the lanes that use this form).  w is formed as
-// min((rc - r) + s, 2s): rc - r is exact for the pairs near the cutoff, so w
-// carries one rounding.  Lanes with w <= 0 (sphere j wholly past rc, masked
-// lanes) give 0.
+//   H = 1/(4r) [ (s/L) z^2 - J(z) ].
+// w is formed as min((rc - r) + s, 2s): rc - r is exact for the pairs near the
+// cutoff, so w carries one rounding.  Lanes with w <= 0 (sphere j wholly past
+// rc, masked lanes) give 0.
 struct CutFar {
     f2 z, w, iL, iU, B;
     bool cx, cy;                      // U' = rc (the cutoff limits the shells)
@@ -245,16 +255,7 @@ __device__ __forceinline__ CutFar hct_cut_far_terms(f2 r, f2 s, float rc, bool u
     const f2 U = add2(L, c.w);
     c.iU = rcp2(U);
     c.z = mul2(c.w, c.iU);
-    const f2 z2 = mul2(c.z, c.z), z3 = mul2(z2, c.z);
-    f2 J = mul2(z3, gb_poly_q2(c.z));
-    if (__any_sync(0xffffffffu, (use0 && c.z.x > GB_POLY_ZJ) || (use1 && c.z.y > GB_POLY_ZJ))) {
-        const f2 Jh = mul2(z3, gb_poly_q_hi2(add2(c.z, F2(-GB_POLY_ZMID))));
-        J = make_float2(c.z.x > GB_POLY_ZJ ? Jh.x : J.x, c.z.y > GB_POLY_ZJ ? Jh.y : J.y);
-        if (__any_sync(0xffffffffu, (use0 && c.z.x > GB_POLY_ZJ2) || (use1 && c.z.y > GB_POLY_ZJ2))) {
-            const f2 Jl = add2(logv(mul2(U, c.iL)), neg2(fma2(F2(0.5f), z2, c.z)));   // ln(U'/L) - z - z^2/2
-            J = make_float2(c.z.x > GB_POLY_ZJ2 ? Jl.x : J.x, c.z.y > GB_POLY_ZJ2 ? Jl.y : J.y);
-        }
-    }
+    const f2 z2 = mul2(c.z, c.z), J = shell_J(c.z, mul2(U, c.iL), use0, use1);
     c.B = fma2(mul2(s, c.iL), z2, neg2(J));
     return c;
 }
@@ -273,9 +274,8 @@ __device__ __forceinline__ f2 hct_cut_far_fr2(f2 r, f2 rinv, f2 s, float rc, boo
     const f2 dH = mul2(mul2(F2(0.25f), rinv), fma2(neg2(c.B), rinv, dB));
     return mul2(neg2(dH), rinv);
 }
-// One direction (descreened atom radius a, descreening sphere s) of every
-// lane of a step in which some sphere crosses rc: disjoint spheres take the
-// restricted form above (the whole sphere while it lies inside the ball, 0
+// One direction (descreened atom radius a, descreening sphere s) per half of
+// a queued pair near rc (see BornCut): disjoint spheres take the restricted form above (the whole sphere while it lies inside the ball, 0
 // once it lies wholly past rc), overlapping ones the general restricted
 // closed form behind a vote.
 __device__ __forceinline__ f2 hct_cut_dir2(f2 r, f2 rinv, f2 a, f2 s, float rc) {
@@ -310,12 +310,9 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
 // tile is the x half's own tile and the y half is below the diagonal (off);
 // mode DY: the tile is the y half's own tile (x half fully on).
 enum { M_FULL = 0, M_DX = 1, M_DY = 2 };
-// Per-block bounds (see block_info): far block; r^2 >= t_near proves the
-// far-field form valid for both directions of a pair.
+// Per-block bounds of the general energy code (see block_info).
 struct BlockInfo {
-    bool far;
-    bool straddle;    // EF_CUT kernels: some pairs of the block on each side of the cutoff
-    float t_near;
+    bool far;         // no pair within the soft repulsion's range
     float skip2;      // EF_STRADDLE blocks: a step whose pairs all have r^2 > skip2 adds nothing
 };
 struct Mask {
@@ -363,116 +360,6 @@ struct Born {
     static constexpr int NJ = 1;      // j-side ones that close pairs add to
     static constexpr bool RADIUS_CUT = true;   // EF_CUT: the cutoff is rgbmax
     static constexpr bool CHAIN = false;
-    struct IState {
-        f2 nx, ny, nz, a, s, s2, hs3;   // nx = -x
-    };
-    struct JState { float x, y, z, a, s, acc; };
-    struct Part {
-        f2 I;
-        __device__ __forceinline__ void zero() { I = F2(0.0f); }
-    };
-    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, IState& st) {
-        float x0, y0, z0, a0, s0, x1, y1, z1, a1, s1;
-        load_xas(A, base, n, i0 + lane, x0, y0, z0, a0, s0);
-        load_xas(A, base, n, i0 + 32 + lane, x1, y1, z1, a1, s1);
-        st.nx = make_float2(-x0, -x1); st.ny = make_float2(-y0, -y1); st.nz = make_float2(-z0, -z1);
-        st.a = make_float2(a0, a1); st.s = make_float2(s0, s1);
-        st.s2 = mul2(st.s, st.s);
-        st.hs3 = mul2(mul2(F2(0.5f), st.s2), st.s);
-    }
-    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, JState& st) {
-        load_xas(A, base, n, j, st.x, st.y, st.z, st.a, st.s);
-        st.acc = 0.0f;
-    }
-    template <int FLAGS, int MODE, bool FAR>
-    static __device__ __forceinline__ void pair(const PairArgs& A, const IState& i, JState& j, Part& p, Mask m,
-                                                const BlockInfo& bi, int, int, int) {
-        const f2 dx = add2(F2(j.x), i.nx), dy = add2(F2(j.y), i.ny), dz = add2(F2(j.z), i.nz);
-        const f2 r2 = safe_r2<MODE>(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), m);
-        // the MUFU estimate's error enters r^-4 four times, and the closed
-        // form cancels its terms about tenfold: 1/r gets a Newton step
-        const f2 rinv = rsqrt2_nr(r2);
-        const f2 rinv2 = mul2(rinv, rinv), rinv4 = mul2(rinv2, rinv2);
-        const float sj2 = j.s * j.s;
-        const float hs3j = 0.5f * sj2 * j.s;
-        const f2 y_ij = mul2(F2(sj2), rinv2), y_ji = mul2(i.s2, rinv2);
-        // EF_STRADDLE: lanes whose sphere lies wholly past rgbmax give 0; a step
-        // with some sphere across it takes the restricted form for every lane
-        bool out_ij0 = false, out_ij1 = false, out_ji0 = false, out_ji1 = false;
-        if (FLAGS & EF_STRADDLE) {
-            const f2 r = mul2(r2, rinv);
-            const float rc = A.rgbmax;
-            out_ij0 = r.x - j.s >= rc; out_ij1 = r.y - j.s >= rc;
-            out_ji0 = r.x - i.s.x >= rc; out_ji1 = r.y - i.s.y >= rc;
-            const bool sh = (!out_ij0 && r.x + j.s > rc) || (!out_ij1 && r.y + j.s > rc) ||
-                            (!out_ji0 && r.x + i.s.x > rc) || (!out_ji1 && r.y + i.s.y > rc);
-            if (__any_sync(0xffffffffu, sh)) {
-                const f2 h_ij = keep<MODE>(hct_cut_dir2(r, rinv, i.a, F2(j.s), rc), m);
-                const f2 h_ji = keep<MODE>(hct_cut_dir2(r, rinv, F2(j.a), i.s, rc), m);
-                p.I = add2(p.I, h_ij);
-                j.acc += h_ji.x + h_ji.y;
-                return;
-            }
-        }
-        // the block bound t_near decides most steps with one compare per lane;
-        // the exact per-direction tests run only on steps where some pair is
-        // closer
-        const float r2min = fminf(r2.x, r2.y);
-        f2 g_ij, g_ji;
-        if (all_far(y_ij, y_ji)) {
-            g_ij = gb_poly_gf2(y_ij);
-            g_ji = gb_poly_gf2(y_ji);
-        } else {
-            g_ij = gb_poly_g2(y_ij);
-            g_ji = gb_poly_g2(y_ji);
-        }
-        f2 h_ij = mul2(F2(hs3j), mul2(rinv4, g_ij));
-        f2 h_ji = mul2(i.hs3, mul2(rinv4, g_ji));
-        if (__any_sync(0xffffffffu, r2min < bi.t_near)) {
-            const f2 r = mul2(r2, rinv);
-            const f2 lim_ij = add2(i.a, F2(j.s)), lim_ji = add2(F2(j.a), i.s);
-            const bool b0 = !far_ok(r.x, lim_ij.x, y_ij.x), b1 = !far_ok(r.y, lim_ij.y, y_ij.y);
-            const bool c0 = !far_ok(r.x, lim_ji.x, y_ji.x), c1 = !far_ok(r.y, lim_ji.y, y_ji.y);
-            if (__any_sync(0xffffffffu, b0 || b1)) {
-                const f2 hc = hct_closed2(r, rinv, i.a, F2(j.s));
-                h_ij = make_float2(b0 ? hc.x : h_ij.x, b1 ? hc.y : h_ij.y);
-            }
-            if (__any_sync(0xffffffffu, c0 || c1)) {
-                const f2 hc = hct_closed2(r, rinv, F2(j.a), i.s);
-                h_ji = make_float2(c0 ? hc.x : h_ji.x, c1 ? hc.y : h_ji.y);
-            }
-        }
-        if (FLAGS & EF_STRADDLE) {   // no sphere across rgbmax: wholly inside or past it
-            h_ij = make_float2(out_ij0 ? 0.0f : h_ij.x, out_ij1 ? 0.0f : h_ij.y);
-            h_ji = make_float2(out_ji0 ? 0.0f : h_ji.x, out_ji1 ? 0.0f : h_ji.y);
-        }
-        h_ij = keep<MODE>(h_ij, m);
-        h_ji = keep<MODE>(h_ji, m);
-        p.I = add2(p.I, h_ij);
-        j.acc += h_ji.x + h_ji.y;
-    }
-    static __device__ __forceinline__ void rotate_data(JState& j, int src) {
-        j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
-        j.a = shfl(j.a, src); j.s = shfl(j.s, src);
-    }
-    static __device__ __forceinline__ void rotate_acc(JState& j, int src) { j.acc = shfl(j.acc, src); }
-    static __device__ __forceinline__ void take_data(JState& j, const JState& d) {
-        j.x = d.x; j.y = d.y; j.z = d.z; j.a = d.a; j.s = d.s;
-    }
-    static __device__ __forceinline__ void fold_i(IState&, long long* sa, int lane, const Part& p) {
-        sa[lane] += fix_i(p.I.x);
-        sa[32 + lane] += fix_i(p.I.y);
-    }
-    // Two atoms at the same position (r = 0; masked pairs read as far first):
-    // r = r^2 / r is NaN, the closed form carries it through U = r + s and
-    // the restricted form of the cutoff through w = r - s^2/r, so both atoms'
-    // sums turn NaN.  One test per block and lane, on the j side, records it
-    // before the fixed-point conversion would hide it.
-    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const JState& st) {
-        if (!isfinite(st.acc) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
-        if (j < n) red_add(&A.I_acc[base + j], fix_i(st.acc));
-    }
-    static __device__ __forceinline__ void flush_sums(const PairArgs&, int, int, const IState&) {}
     static __device__ __forceinline__ void flush_i(const PairArgs& A, int64_t base, int n, int i0, int lane,
                                                    long long* sa) {
         if (i0 + lane < n) red_add(&A.I_acc[base + i0 + lane], sa[lane]);
@@ -698,124 +585,11 @@ struct Chain {
     static constexpr int NJ = 3;
     static constexpr bool RADIUS_CUT = true;   // EF_CUT: the cutoff is rgbmax
     static constexpr bool CHAIN = true;
-    struct IState {
-        f2 nx, ny, nz, a, s, s2, hs3, c;
-    };
-    struct JState { float x, y, z, a, s, c, fx, fy, fz; };
-    struct Part {
-        f2 sx, sy, sz;
-        __device__ __forceinline__ void zero() { sx = sy = sz = F2(0.0f); }
-    };
     static __device__ __forceinline__ void load_one(const PairArgs& A, int64_t base, int n, int i, float& x,
                                                     float& y, float& z, float& a, float& s, float& c) {
         load_xas(A, base, n, i, x, y, z, a, s);
         c = (i < n) ? __ldcg(&A.cc[base + i]) : 0.0f;
     }
-    static __device__ __forceinline__ void load_i(const PairArgs& A, int64_t base, int n, int i0, int lane, IState& st) {
-        float x0, y0, z0, a0, s0, c0, x1, y1, z1, a1, s1, c1;
-        load_one(A, base, n, i0 + lane, x0, y0, z0, a0, s0, c0);
-        load_one(A, base, n, i0 + 32 + lane, x1, y1, z1, a1, s1, c1);
-        st.nx = make_float2(-x0, -x1); st.ny = make_float2(-y0, -y1); st.nz = make_float2(-z0, -z1);
-        st.a = make_float2(a0, a1); st.s = make_float2(s0, s1); st.c = make_float2(c0, c1);
-        st.s2 = mul2(st.s, st.s);
-        st.hs3 = mul2(mul2(F2(0.5f), st.s2), st.s);
-    }
-    static __device__ __forceinline__ void load_j(const PairArgs& A, int64_t base, int n, int j, JState& st) {
-        load_one(A, base, n, j, st.x, st.y, st.z, st.a, st.s, st.c);
-        st.fx = st.fy = st.fz = 0.0f;
-    }
-    template <int FLAGS, int MODE, bool FAR>
-    static __device__ __forceinline__ void pair(const PairArgs& A, const IState& i, JState& j, Part& p, Mask m,
-                                                const BlockInfo& bi, int, int, int) {
-        const f2 dx = add2(F2(j.x), i.nx), dy = add2(F2(j.y), i.ny), dz = add2(F2(j.z), i.nz);
-        const f2 r2 = safe_r2<MODE>(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), m);
-        const f2 rinv = rsqrt2(r2);
-        const f2 rinv2 = mul2(rinv, rinv);
-        const float sj2 = j.s * j.s;
-        const float hs3j = 0.5f * sj2 * j.s;
-        const f2 y_ij = mul2(F2(sj2), rinv2), y_ji = mul2(i.s2, rinv2);
-        // EF_STRADDLE: as in Born; a lane with one direction wholly past rgbmax
-        // has the other across it or past it too
-        bool out0 = false, out1 = false;
-        if (FLAGS & EF_STRADDLE) {
-            const f2 r = mul2(r2, rinv);
-            const float rc = A.rgbmax;
-            out0 = r.x - j.s >= rc && r.x - i.s.x >= rc;
-            out1 = r.y - j.s >= rc && r.y - i.s.y >= rc;
-            const bool sh = (!out0 && (r.x + j.s > rc || r.x + i.s.x > rc)) ||
-                            (!out1 && (r.y + j.s > rc || r.y + i.s.y > rc));
-            if (__any_sync(0xffffffffu, sh)) {
-                const f2 fr = keep<MODE>(fma2(i.c, hct_cut_dir_fr2(r, rinv, i.a, F2(j.s), rc),
-                                              mul2(F2(j.c), hct_cut_dir_fr2(r, rinv, F2(j.a), i.s, rc))), m);
-                p.sx = fma2(fr, dx, p.sx); p.sy = fma2(fr, dy, p.sy); p.sz = fma2(fr, dz, p.sz);
-                j.fx = fmaf(fr.y, dx.y, fmaf(fr.x, dx.x, j.fx));
-                j.fy = fmaf(fr.y, dy.y, fmaf(fr.x, dy.x, j.fy));
-                j.fz = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, j.fz));
-                return;
-            }
-        }
-        // c_i s_j^3/2 h(y_ij) + c_j s_i^3/2 h(y_ji), times r^-6
-        const float r2min = fminf(r2.x, r2.y);
-        f2 p_ij, p_ji;
-        if (all_far(y_ij, y_ji)) {
-            p_ij = gb_poly_hf2(y_ij);
-            p_ji = gb_poly_hf2(y_ji);
-        } else {
-            p_ij = gb_poly_h2(y_ij);
-            p_ji = gb_poly_h2(y_ji);
-        }
-        const f2 t_ij = mul2(mul2(i.c, F2(hs3j)), p_ij);
-        const f2 t_ji = mul2(mul2(F2(j.c), i.hs3), p_ji);
-        const f2 rinv6 = mul2(rinv2, mul2(rinv2, rinv2));
-        f2 fr = mul2(add2(t_ij, t_ji), rinv6);
-        if (__any_sync(0xffffffffu, r2min < bi.t_near)) {
-            const f2 r = mul2(r2, rinv);
-            const f2 lim_ij = add2(i.a, F2(j.s)), lim_ji = add2(F2(j.a), i.s);
-            const bool b0 = !far_ok(r.x, lim_ij.x, y_ij.x), b1 = !far_ok(r.y, lim_ij.y, y_ij.y);
-            const bool c0 = !far_ok(r.x, lim_ji.x, y_ji.x), c1 = !far_ok(r.y, lim_ji.y, y_ji.y);
-            f2 fb = mul2(t_ij, rinv6), fc = mul2(t_ji, rinv6);
-            if (__any_sync(0xffffffffu, b0 || b1)) {
-                const f2 hc = mul2(i.c, hct_closed_fr2(r, rinv, i.a, F2(j.s)));
-                fb = make_float2(b0 ? hc.x : fb.x, b1 ? hc.y : fb.y);
-            }
-            if (__any_sync(0xffffffffu, c0 || c1)) {
-                const f2 hc = mul2(F2(j.c), hct_closed_fr2(r, rinv, F2(j.a), i.s));
-                fc = make_float2(c0 ? hc.x : fc.x, c1 ? hc.y : fc.y);
-            }
-            const f2 fbc = add2(fb, fc);
-            fr = make_float2(b0 || c0 ? fbc.x : fr.x, b1 || c1 ? fbc.y : fr.y);
-        }
-        if (FLAGS & EF_STRADDLE) fr = make_float2(out0 ? 0.0f : fr.x, out1 ? 0.0f : fr.y);
-        fr = keep<MODE>(fr, m);
-        p.sx = fma2(fr, dx, p.sx); p.sy = fma2(fr, dy, p.sy); p.sz = fma2(fr, dz, p.sz);
-        j.fx = fmaf(fr.y, dx.y, fmaf(fr.x, dx.x, j.fx));
-        j.fy = fmaf(fr.y, dy.y, fmaf(fr.x, dy.x, j.fy));
-        j.fz = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, j.fz));
-    }
-    static __device__ __forceinline__ void rotate_data(JState& j, int src) {
-        j.x = shfl(j.x, src); j.y = shfl(j.y, src); j.z = shfl(j.z, src);
-        j.a = shfl(j.a, src); j.s = shfl(j.s, src); j.c = shfl(j.c, src);
-    }
-    static __device__ __forceinline__ void rotate_acc(JState& j, int src) {
-        j.fx = shfl(j.fx, src); j.fy = shfl(j.fy, src); j.fz = shfl(j.fz, src);
-    }
-    static __device__ __forceinline__ void take_data(JState& j, const JState& d) {
-        j.x = d.x; j.y = d.y; j.z = d.z; j.a = d.a; j.s = d.s; j.c = d.c;
-    }
-    static __device__ __forceinline__ void fold_i(IState&, long long* sa, int lane, const Part& p) {
-        sa[lane] -= fix(p.sx.x); sa[32 + lane] -= fix(p.sx.y);
-        sa[64 + lane] -= fix(p.sy.x); sa[96 + lane] -= fix(p.sy.y);
-        sa[128 + lane] -= fix(p.sz.x); sa[160 + lane] -= fix(p.sz.y);
-    }
-    static __device__ __forceinline__ void flush_j(const PairArgs& A, int64_t base, int n, int j, const JState& st) {
-        if (j < n) {
-            const int64_t g = base + j;
-            red_add(&A.F_acc[g], fix(st.fx));
-            red_add(&A.F_acc[A.N + g], fix(st.fy));
-            red_add(&A.F_acc[2 * A.N + g], fix(st.fz));
-        }
-    }
-    static __device__ __forceinline__ void flush_sums(const PairArgs&, int, int, const IState&) {}
     static __device__ __forceinline__ void flush_i(const PairArgs& A, int64_t base, int n, int i0, int lane,
                                                    long long* sa) {
 #pragma unroll
@@ -861,8 +635,7 @@ __device__ __forceinline__ void run_tile(const PairArgs& A, const typename P::IS
     // a DX block pairs the x half with its own tile: only steps 1 .. 16 carry
     // pairs (js enters rotated by one and leaves rotated by 17)
     constexpr int K0 = (MODE == M_DX) ? 1 : 0, K1 = (MODE == M_DX) ? 17 : 32;
-    // straddling blocks carry the long restricted-integral code: not unrolled,
-    // so that it fits the instruction cache
+    // with steps left out the loop is not worth unrolling
     constexpr int U = (FLAGS & EF_STRADDLE) ? 1 : 2;
 #pragma unroll U
     for (int k = K0; k < K1; ++k) {
@@ -885,14 +658,6 @@ __device__ __forceinline__ void run_tile(const PairArgs& A, const typename P::IS
     }
 }
 
-// Classification of a block (super-row K, tile J) from the bounding boxes of
-// its tiles (lo.xyz with max a, hi.xyz with max s, from k_tile_boxes).  The
-// block is "far" when the boxes prove, for every pair, r >= a_i + s_j
-// (disjoint spheres), (s/r)^2 <= YFAR (short polynomial exact to FP32) and
-// r >= the soft-repulsion range.  Otherwise r^2 >= t_near proves both
-// directions of a pair disjoint with (s/r)^2 <= YMAX (far-field form valid),
-// so only steps with a closer pair need the exact tests.  Without boxes
-// nothing is proven.
 // Bounds between the box of super-row K (tiles 2K, 2K+1) and the box of tile
 // J: least and greatest distance squared, largest a and largest s of both.
 struct BoxPair {
@@ -945,37 +710,18 @@ __device__ __forceinline__ void cut_class(const PairArgs& A, bool radius_cut, co
     }
 }
 
-template <class P>
+// Bounds of a block from the bounding boxes of its tiles (lo.xyz with max a,
+// hi.xyz with max s, from k_tile_boxes); without boxes nothing is proven.
 __device__ __forceinline__ BlockInfo block_info(const PairArgs& A, int r, int K, int J, int nb) {
     BlockInfo bi;
-    bi.skip2 = INFINITY;
-    if (!A.boxes) {   // nothing proven: near, and straddling when a cutoff is applied
-        bi.far = false;
-        bi.straddle = true;
-        bi.t_near = INFINITY;
-        return bi;
-    }
-    const int t0 = A.tile_off[r];
-    const float4 jl = __ldcg(&A.boxes[2 * (t0 + J)]), jh = __ldcg(&A.boxes[2 * (t0 + J) + 1]);
-    float4 ih;
-    const float4 il = row_box_lo(A, t0, K, nb, &ih);
-    const BoxPair b = box_pair(il, ih, jl, jh);
-    const float as = b.amax + b.smax;
-    bi.far = b.rmin2 >= as * as && b.smax * b.smax <= GB_POLY_YFAR * b.rmin2;
-    if (A.rep_k != 0.0f) bi.far = bi.far && b.rmin2 >= A.rep_sigma * A.rep_sigma;
-    // thresholds rounded up a little, so that rounding in r^2 cannot admit a
-    // pair the exact test would reject
-    bi.t_near = 1.0001f * fmaxf(as * as, b.smax * b.smax * (1.0f / GB_POLY_YMAX));
-    // EF_CUT kernels: the block's cutoff class, and the reach past which a
-    // pair adds exact zeros (Born and chain passes r >= rgbmax + s for both
-    // spheres, energy pass r > max(cut, rep_sigma))
-    bool in;
-    cut_class(A, P::RADIUS_CUT, b, in, bi.straddle);
-    if (P::RADIUS_CUT) {
-        const float reach = A.rgbmax + b.smax;
-        bi.skip2 = 1.001f * reach * reach;
-    } else {
-        bi.skip2 = 1.001f * A.e_range2;
+    bi.far = A.rep_k == 0.0f;
+    bi.skip2 = A.boxes ? 1.001f * A.e_range2 : INFINITY;
+    if (!bi.far && A.boxes) {
+        const int t0 = A.tile_off[r];
+        const float4 jl = __ldcg(&A.boxes[2 * (t0 + J)]), jh = __ldcg(&A.boxes[2 * (t0 + J) + 1]);
+        float4 ih;
+        const float4 il = row_box_lo(A, t0, K, nb, &ih);
+        bi.far = box_pair(il, ih, jl, jh).rmin2 >= A.rep_sigma * A.rep_sigma;
     }
     return bi;
 }
@@ -1025,6 +771,23 @@ __device__ __forceinline__ f2 screen_r2(f2 r2, Mask m, float t, unsigned bit, un
         my |= cy ? bit : 0u;
     }
     return make_float2((DROP && cx) || !m.x ? FAR_R2 : r2.x, (DROP && cy) || !m.y ? FAR_R2 : r2.y);
+}
+
+// Bounds on r^2 in a block that straddles the Born-radius cutoff: pairs from
+// close to in are as without a cutoff, pairs from out on add exact zeros.
+struct Ring { float close, in, out; };
+__device__ __forceinline__ Ring ring_of(const PairArgs& A, float close, float smax) {
+    const float outer = A.rgbmax + smax, inner = fmaxf(A.rgbmax - smax, 0.0f);
+    return Ring{close, 0.999f * inner * inner, 1.001f * outer * outer};
+}
+// The same screen with a ring: the other pairs read as far, and those before
+// out (or NaN) set their bit.
+template <int MODE, bool NEAR, bool DROP>
+__device__ __forceinline__ f2 screen_r2(f2 r2, Mask m, Ring g, unsigned bit, unsigned& mx, unsigned& my) {
+    const bool kx = r2.x >= g.close && r2.x < g.in, ky = r2.y >= g.close && r2.y < g.in;
+    mx |= !kx && !(r2.x >= g.out) && m.x ? bit : 0u;
+    my |= !ky && !(r2.y >= g.out) && m.y ? bit : 0u;
+    return make_float2(kx && m.x ? r2.x : FAR_R2, ky && m.y ? r2.y : FAR_R2);
 }
 
 // The staged tile of a warp: j atoms (twice, see stage()), what close pairs
@@ -1097,6 +860,7 @@ __device__ __forceinline__ float staged_bound(const Slot<W>& S, int lane) {
 // --- Born integrals --------------------------------------------------------------------
 template <int NW>
 struct BornY {
+    static constexpr bool CUT = false;
     static constexpr int ATOMS = 64 * NW, NQ = Born::NQ, NJ = Born::NJ, UNROLL = NW == 2 ? 2 : 4;
     struct I { f2 nx[NW], ny[NW], nz[NW], s2[NW], hs3[NW]; };
     typedef float B;                                   // staged j values: x, y, z, s^2 | s^3 / 2
@@ -1132,9 +896,9 @@ struct BornY {
 #pragma unroll
         for (int q = 0; q < NW; ++q) p.s[q] = F2(0.0f);
     }
-    template <int MODE = M_FULL, bool NEAR = false>
+    template <int MODE = M_FULL, bool NEAR = false, class T = float>
     static __device__ __forceinline__ void step(const PairArgs&, const I& i, float4 v, B b, J& j, Part& p,
-                                                Mask m = Mask{true, true}, float t = 0.0f, unsigned bit = 0,
+                                                Mask m = Mask{true, true}, T t = T(), unsigned bit = 0,
                                                 unsigned* mk = nullptr) {
 #pragma unroll
         for (int q = 0; q < NW; ++q) {
@@ -1310,6 +1074,7 @@ struct ForceSums {
 template <int NW>
 struct ChainY : ForceSums<NW> {
     typedef ForceSums<NW> F;
+    static constexpr bool CUT = false;
     static constexpr int ATOMS = 64 * NW, NQ = Chain::NQ, NJ = Chain::NJ, UNROLL = NW == 2 ? 1 : 4;
     struct I { f2 nx[NW], ny[NW], nz[NW], s2[NW], hs3[NW], c[NW]; };
     typedef float2 B;                                  // staged j values: x, y, z, s^2 | s^3 / 2, c
@@ -1338,9 +1103,9 @@ struct ChainY : ForceSums<NW> {
         float2 as;
         load(A, base, n, j, v, b, as);
     }
-    template <int MODE = M_FULL, bool NEAR = false>
+    template <int MODE = M_FULL, bool NEAR = false, class T = float>
     static __device__ __forceinline__ void step(const PairArgs&, const I& i, float4 v, B b, typename F::J& j,
-                                                typename F::Part& p, Mask m = Mask{true, true}, float t = 0.0f,
+                                                typename F::Part& p, Mask m = Mask{true, true}, T t = T(),
                                                 unsigned bit = 0, unsigned* mk = nullptr) {
 #pragma unroll
         for (int q = 0; q < NW; ++q) {
@@ -1446,6 +1211,7 @@ struct ChainU : ForceSums<NW> {
 template <int NW, int FLAGS>
 struct EnergyW : ForceSums<NW> {
     typedef ForceSums<NW> F;
+    static constexpr bool CUT = false;
     static constexpr int ATOMS = 64 * NW, NQ = Energy::NQ, NJ = Energy::NJ, UNROLL = NW == 2 ? 1 : 4;
     struct I { f2 nx[NW], ny[NW], nz[NW], Q[NW], R[NW], nh[NW]; };
     typedef float2 B;                                  // staged j values: x, y, z, q | R, h
@@ -1645,9 +1411,28 @@ __device__ __noinline__ int close_pairs(const PairArgs& A, int slot, int row, un
     return total;
 }
 
-template <class W, int MODE, bool NEAR>
+// The bound of a near tile: that of its boxes, or from the staged atoms.
+template <class W, bool CUT = W::CUT>
+struct NearBound { typedef float T; };
+template <class W>
+struct NearBound<W, true> { typedef Ring T; };
+template <class W>
+__device__ __forceinline__ typename NearBound<W>::T near_bound(const PairArgs& A, const Slot<W>& S, float t, float smax, int lane) {
+    if constexpr (W::CUT) {
+        if (!A.boxes) {
+            t = staged_bound(S, lane);
+            smax = fmaxf(S.ja[lane].y, fmaxf(S.i2[lane].y, S.i2[32 + lane].y));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+        }
+        return ring_of(A, t, smax);
+    } else {
+        return A.boxes ? t : W::bound(A, S, lane);
+    }
+}
+template <class W, int MODE, bool NEAR, class T>
 __device__ __forceinline__ void near_tile(const PairArgs& A, const typename W::I& is, const Slot<W>& S,
-                                            typename W::J& js, typename W::Part& p, float t, unsigned* mk, int lane) {
+                                          typename W::J& js, typename W::Part& p, T t, unsigned* mk, int lane) {
     // a DX block pairs the x half with its own tile: only steps 1 .. 16 carry pairs
     constexpr int K0 = (MODE == M_DX) ? 1 : 0, K1 = (MODE == M_DX) ? 17 : 32;
     const int next = (lane + 1) & 31;
@@ -1662,7 +1447,8 @@ __device__ __forceinline__ void near_tile(const PairArgs& A, const typename W::I
 // t: of lane c the bound below which pairs of column J0 + c are close.  DEFER
 // (one column): the close pairs stay in the queue, their number is returned.
 template <class W, bool CLOSE, bool DEFER = false>
-__device__ __noinline__ int walk_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot) {
+__device__ __noinline__ int walk_near(const PairArgs& A, int r, int K, int J0, unsigned todo, float t, int slot,
+                                      float smax = 0.0f) {
     const int lane = threadIdx.x & 31;
     slot = __shfl_sync(0xffffffffu, slot, 0);
     r = __shfl_sync(0xffffffffu, r, 0);
@@ -1687,8 +1473,7 @@ __device__ __noinline__ int walk_near(const PairArgs& A, int r, int K, int J0, u
         S.jb[lane] = S.jb[32 + lane] = b;
         S.ja[lane] = as;
         __syncwarp();
-        float tc = __shfl_sync(0xffffffffu, t, c);
-        if (!A.boxes) tc = W::bound(A, S, lane);
+        typename NearBound<W>::T tc = near_bound(A, S, __shfl_sync(0xffffffffu, t, c), __shfl_sync(0xffffffffu, smax, c), lane);
         typename W::J js;
         typename W::Part p;
         W::zero(js, p);
@@ -1713,8 +1498,8 @@ __device__ __noinline__ int walk_near(const PairArgs& A, int r, int K, int J0, u
     }
 }
 
-// The same row by the general pair code: blocks that straddle a cutoff
-// (EF_STRADDLE), and passes that want energies or dE/dq.
+// The same row by the general pair code of the energy pass: blocks that
+// straddle the pair cutoff (EF_STRADDLE), and passes that want energies or dE/dq.
 template <class P, int FLAGS>
 __device__ __noinline__ void walk_general(const PairArgs& A, int r, int K, int J0, unsigned todo, int slot) {
     extern __shared__ __align__(16) unsigned char s_mem[];
@@ -1732,7 +1517,7 @@ __device__ __noinline__ void walk_general(const PairArgs& A, int r, int K, int J
         P::load_j(A, base, n, 32 * J + ((lane + (dx ? 1 : 0)) & 31), js);
         typename P::Part ip;
         ip.zero();
-        const BlockInfo bi = block_info<P>(A, r, K, J, nb);
+        const BlockInfo bi = block_info(A, r, K, J, nb);
         if (J >= 2 * K + 2) {
             if (!(FLAGS & EF_STRADDLE) && bi.far) run_tile<P, FLAGS, M_FULL, true>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
             else run_tile<P, FLAGS, M_FULL, false>(A, is, js, ip, bi, 64 * K, 32 * J, lane, next);
@@ -1746,6 +1531,51 @@ __device__ __noinline__ void walk_general(const PairArgs& A, int r, int K, int J
     }
     P::flush_sums(A, r, lane, is);
 }
+
+// --- blocks that straddle the Born-radius cutoff --------------------------------------
+// Pairs wholly inside the cutoff take the near form, pairs past its reach are
+// left out, and the close ones and those whose sphere may cross it (see Ring)
+// are queued and evaluated exactly, 32 at a time.  The restricted integrals
+// cost ten times the near form and the sphere about the cutoff is thin (two
+// times the largest s), but nearly every step of 64 pairs has a pair in it:
+// taking the restricted form for all lanes of such steps bound the Born and
+// chain passes, 641 and 980 us at 100,000 atoms and 12 A against 483 and 733
+// now (25 A: 1600 and 2550 against 1186 and 1759).  Queueing all pairs in
+// reach and none in the near form: 767 and 965 (25 A: 1856 and 2668).
+struct BornCut : BornY<1> {
+    static constexpr bool CUT = true;
+    static __device__ __forceinline__ void close(const PairArgs& A, const Slot<BornCut>& S, long long* sa, int i, int j,
+                                                 bool valid, int, int) {
+        const float4 xi = S.i4[i], xj = S.j4[j];
+        const float2 ai = S.i2[i], aj = S.ja[j];
+        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+        const f2 r2 = F2(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        const f2 rinv = rsqrt2_nr(r2), r = mul2(r2, rinv);
+        const f2 h = hct_cut_dir2(r, rinv, make_float2(ai.x, aj.x), make_float2(aj.y, ai.y), A.rgbmax);
+        if (!valid) return;
+        if (!isfinite(h.x + h.y) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
+        long long* const to[2] = {&sa[i], &S.jac[j]};
+        const long long v[2] = {fix_i(h.x), fix_i(h.y)};
+        shared_add(to, v);
+    }
+};
+struct ChainCut : ChainY<1> {
+    static constexpr bool CUT = true;
+    static __device__ __forceinline__ void close(const PairArgs& A, const Slot<ChainCut>& S, long long* sa, int i, int j,
+                                                 bool valid, int, int) {
+        const float4 xi = S.i4[i], xj = S.j4[j];
+        const float2 ai = S.i2[i], aj = S.ja[j];
+        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+        const f2 r2 = F2(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        const f2 rinv = rsqrt2_nr(r2), r = mul2(r2, rinv);
+        const f2 h = hct_cut_dir_fr2(r, rinv, make_float2(ai.x, aj.x), make_float2(aj.y, ai.y), A.rgbmax);
+        if (valid) F::add_close(sa, S.jac, i, j, fmaf(xi.w, h.x, S.jb[j].y * h.y), dx, dy, dz);
+    }
+};
+template <class P>
+struct CutForm { typedef BornCut W; };
+template <>
+struct CutForm<Chain> { typedef ChainCut W; };
 
 // Form of a block (see above) from the bounds of its boxes.
 template <class P, int FLAGS>
@@ -1832,7 +1662,7 @@ __device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, int s
         const int J0 = t.z + s0, m = min(32, t.w - s0), J = J0 + lane;
         int tier[2] = {0, 0};
         bool in[2] = {true, true}, straddle[2] = {CUT, CUT};
-        float bound[2] = {0.0f, 0.0f};
+        float bound[2] = {0.0f, 0.0f}, smax[2] = {0.0f, 0.0f};
         if (A.boxes && lane < m) {
             const int t0 = A.tile_off[r];
             const float4 jl = __ldcg(&A.boxes[2 * (t0 + J)]), jh = __ldcg(&A.boxes[2 * (t0 + J) + 1]);
@@ -1845,6 +1675,7 @@ __device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, int s
                 tier[h] = row_tier<P, FLAGS>(A, b);
                 bound[h] = P::RADIUS_CUT ? close_bound(b.amax, b.smax) : A.rep_sigma * A.rep_sigma;
                 if (CUT) cut_class(A, P::RADIUS_CUT, b, in[h], straddle[h]);
+                smax[h] = b.smax;
             }
         }
         const unsigned all = m == 32 ? 0xffffffffu : (1u << m) - 1u;
@@ -1869,7 +1700,9 @@ __device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, int s
             if (!((sel >> h) & 1) || 2 * K >= nb || !todo) continue;
             used |= 1u << h;
             const unsigned st = CUT ? todo & __ballot_sync(0xffffffffu, straddle[h]) : 0u, rest = todo & ~st;
-            if constexpr (CUT) {
+            if constexpr (CUT && P::RADIUS_CUT) {
+                if (st) walk_near<typename CutForm<P>::W, true>(A, r, K, J0, st, bound[h], slot, smax[h]);
+            } else if constexpr (CUT) {
                 if (st) walk_general<P, FLAGS | EF_STRADDLE>(A, r, K, J0, st, slot);
             }
             if constexpr (GENERAL) {
