@@ -40,10 +40,10 @@ MD_PER_STEP = 100          # MD steps per bench step (one exchange period)
 MC_EVERY, EX_EVERY = 10, 100
 FP32_LANES = 128           # FP32 lanes per SM
 # Algorithmic FP32 flops per unordered pair and pass (FMA = 2, add / mul = 1;
-# MUFU ops counted apart), counted on the far-field arithmetic every disjoint
-# pair needs (short polynomials); pairs in near blocks cost more, so these
-# figures are a lower bound of the FP32 work done.
-FLOPS_PER_PAIR = {"born": 34.0, "energy": 43.0, "chain": 51.0}
+# MUFU ops counted apart), counted on the cheapest form a pair can take
+# (distant blocks); pairs in nearer blocks cost more, so these figures are a
+# lower bound of the FP32 work done.
+FLOPS_PER_PAIR = {"born": 21.0, "energy": 43.0, "chain": 34.0}
 MUFU_PER_PAIR = {"born": 1, "energy": 3, "chain": 1}
 PASS_NAMES = ["born", "energy", "chain"]
 

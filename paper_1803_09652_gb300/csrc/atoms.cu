@@ -151,7 +151,8 @@ __global__ void k_advance_counters(u64* ctr, u64 steps, u64 attempts) {
 // with the site rows
 //   phi_k = sum_{j != k} q_j (k_c / r_kj - tau k_e / f_kj) - tau k_e q_k / R_k
 // and the site-site block A_kl = k_c / r_kl - tau k_e / f_kl (k != l),
-// A_kk = -tau k_e / R_k.  Terms in FP32, sums and the decision in FP64.
+// A_kk = -tau k_e / R_k.  Row terms in FP32 with compensated sums (Sum2), the
+// rest and the decision in FP64.
 // Stage 1 (k_mc_rows) splits each replica's atoms into MC_CHUNK-atom slices,
 // one block per (slice, replica), and stores per-slice partial rows; stage 2
 // (k_mc_decide) adds the slices in a fixed order, adds the site block, and

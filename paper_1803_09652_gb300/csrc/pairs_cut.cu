@@ -19,7 +19,7 @@ namespace gbk {
 
 namespace {
 
-constexpr int RUN = 4;           // blocks per task at most (100,000 atoms, 12 A: 1.97 ms; 8: 2.05, 16: 2.27)
+constexpr int RUN = 4;           // blocks per task at most (100,000 atoms, 12 A: 1.64 ms; 8: 1.73; at 25 A 3.97 and 3.94)
 
 __global__ void k_list_reset(int* ctr) {
     pdl_enter();
