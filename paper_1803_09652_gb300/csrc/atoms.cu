@@ -151,8 +151,8 @@ __global__ void k_advance_counters(u64* ctr, u64 steps, u64 attempts) {
 // with the site rows
 //   phi_k = sum_{j != k} q_j (k_c / r_kj - tau k_e / f_kj) - tau k_e q_k / R_k
 // and the site-site block A_kl = k_c / r_kl - tau k_e / f_kl (k != l),
-// A_kk = -tau k_e / R_k.  Row terms in FP32 with compensated sums (Sum2), the
-// rest and the decision in FP64.
+// A_kk = -tau k_e / R_k.  Row terms in FP32, their sums as exact as in FP64 (RowSum),
+// the rest and the decision in FP64.
 // Stage 1 (k_mc_rows) splits each replica's atoms into MC_CHUNK-atom slices,
 // one block per (slice, replica), and stores per-slice partial rows; stage 2
 // (k_mc_decide) adds the slices in a fixed order, adds the site block, and
@@ -234,22 +234,32 @@ __device__ __forceinline__ float mc_self_term(float Rk, float tke, float kc, flo
     return -t / Rk;
 }
 
-// Sum of FP32 terms to about 2^-40 of its size without FP64, which this GPU
-// issues at 1/64 of the FP32 rate: s carries the rounded sum and c the exact
-// rounding errors of its additions (Knuth's two-sum).
-struct Sum2 {
-    float s = 0.0f, c = 0.0f;
-    __device__ __forceinline__ void add(float x, float low = 0.0f) {
-        const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
-        c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)) + low;
-        s = t;
+// Sum of FP32 terms at least as exact as one in FP64, without the FP64 pipe, which
+// this GPU issues at 1/64 of the FP32 rate: s carries the rounded sum, c the
+// rounding errors of its additions and d those of the additions to c, each of
+// them exact (Knuth's two-sum).  A sum that meets an infinity or a NaN is what
+// s holds, the same as in FP64: the errors of its additions are NaN by then.
+struct RowSum {
+    float s = 0.0f, c = 0.0f, d = 0.0f;
+    static __device__ __forceinline__ float two_sum(float& a, float x) {
+        const float t = __fadd_rn(a, x), z = __fsub_rn(t, a);
+        const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(x, z));
+        a = t;
+        return err;
     }
-    // + (h + l) a, with the product's rounding error
+    __device__ __forceinline__ void add_low(float x) { d += two_sum(c, x); }
+    __device__ __forceinline__ void add(float x) { add_low(two_sum(s, x)); }
+    // + (h + l) a, with the products' rounding errors
     __device__ __forceinline__ void add_product(float h, float l, float a) {
-        const float p = __fmul_rn(h, a);
-        add(p, fmaf(l, a, fmaf(h, a, -p)));
+        const float p = __fmul_rn(h, a), q = __fmul_rn(l, a);
+        add(p);
+        add_low(fmaf(h, a, -p));
+        add_low(q);
+        d += fmaf(l, a, -q);
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    __device__ __forceinline__ double value() const {
+        return isfinite(s) ? (double)s + ((double)c + (double)d) : (double)s;
+    }
 };
 
 // Rows phi of `count` site atoms (replica-local index idx(k)) over the slice
@@ -261,7 +271,8 @@ struct Sum2 {
 // Bound by the pair term's FP32 and MUFU instructions, about 30 a term.  As
 // one warp a site atom with FP64 sums per lane and an FP64 shuffle tree, the
 // FP64 pipe took six times as long as the terms: 530 us for 4 x 25000 atoms
-// and their 620 site atoms a replica.
+// and their 620 site atoms a replica.  The third word of the sums is 4 % of
+// that sweep (305 us a call, 293 with two words, 708 with FP64).
 template <class Idx>
 __device__ __forceinline__ void mc_rows_slice(const MCArgs& A, int64_t base, int j0, int j1, int count, Idx idx,
                                               double* out) {
@@ -285,7 +296,7 @@ __device__ __forceinline__ void mc_rows_slice(const MCArgs& A, int64_t base, int
         const float4 xk = A.xyzq[base + lk];
         const float2 Rk = mc_Rh(A, base + lk);
         const float self = mc_self_term(Rk.x, tke, kc, keo, kap);
-        Sum2 sum;
+        RowSum sum;
         const int end = min(nj, (part + 1) * seg);
 #pragma unroll 4
         for (int j = part * seg; j < end; ++j) {
@@ -496,10 +507,11 @@ __global__ void __launch_bounds__(256) k_sweep_rows(MCArgs A) {
 
 // One block a replica; the visits follow one another, so what a visit waits
 // for is kept short: the numbers of all visits are drawn at once beforehand
-// (their order, proposals and Metropolis thresholds -kT ln u depend on no
-// decision), coordinates, radii and charges of the listed atoms stand in shared
-// memory, sums over the rows use Sum2 instead of FP64, and an accepted move
-// updates only the rows of sites still to be visited.
+// (their order, their proposals and the uniform numbers of the decisions depend
+// on no decision), coordinates, radii and charges of the listed atoms stand in
+// shared memory, an accepted move updates only the rows of sites still to be
+// visited, and those updates are RowSums; the change of energy itself, a sum of
+// at most 128^2 terms, and the decision stay in FP64.
 constexpr int SWEEP_THREADS = 1024;
 __global__ void __launch_bounds__(SWEEP_THREADS) k_sweep_decide(MCArgs A) {
     pdl_enter();
@@ -614,7 +626,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS) k_sweep_decide(MCArgs A) {
                 for (int m = m0 + lane; m < m1; m += 32) {
                     const float4 xm = s_x[m];
                     const float2 Rm = s_R[m];
-                    Sum2 d;
+                    RowSum d;
                     for (int a = 0; a < na; ++a) {
                         float Ama;
                         if (L.atom[a0 + a] == L.atom[m]) {         // an atom of both sites
