@@ -112,7 +112,9 @@ int gb_sync_status(gb_ctx* ctx, void* stream);
  * atoms) per warp task of the static task list (a pass with a cutoff walks
  * its neighbour list instead, in runs of up to 4 blocks).  gb_autotune times
  * the candidates and register caps pass by pass on the given inputs and
- * keeps the fastest; gb_set_tiles forces one. */
+ * keeps the fastest; gb_set_tiles forces one.  Neither tiles nor caps reach
+ * the evaluations and MD segments that run in one launch (small batches); they
+ * count for the others on the same context, those with energies or dE/dq. */
 int gb_autotune(gb_ctx* ctx, const float* xyzq, const float* rad_screen, void* stream);
 int gb_set_tiles(gb_ctx* ctx, int32_t warps_per_block, int32_t tiles_per_task);
 /* Register cap of the pair kernel of one pass (0 Born radii, 1 energy and
@@ -380,7 +382,9 @@ int gb_md_segment_host(gb_ctx* ctx, gb_md_state* state, const gb_sites* sites, i
  * buffers and the state struct are put back as they were before the call
  * returns; the chosen caps stay on the context (gb_get_reg_caps).  Needs
  * forces at the incoming coordinates (after gb_md_init).  Allocates a copy
- * of the state.  GB_ERR_INVALID_ARG for trial_steps outside 1..100000. */
+ * of the state.  Where the segment runs in one launch (a small batch, or the
+ * persistent kernel) it reads no caps, and the call leaves them as they are.
+ * GB_ERR_INVALID_ARG for trial_steps outside 1..100000. */
 int gb_autotune_md(gb_ctx* ctx, gb_md_state* state, const gb_sites* sites, int64_t trial_steps, void* stream);
 
 /* Allocation-free energy / force evaluation of ONE molecule.

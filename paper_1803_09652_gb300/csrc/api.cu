@@ -1307,6 +1307,9 @@ extern "C" int gb_autotune_md(gb_ctx* c, gb_md_state* st, const gb_sites* sites,
     if (rc) return rc;
     if (sites && (rc = check_sites(c, sites))) return rc;
     if (trial_steps < 1 || trial_steps > 100000) return fail(c, GB_ERR_INVALID_ARG, "trial_steps must be 1..100000");
+    // segments that run in one launch read no caps: a choice among them would be
+    // noise, and other calls on the context would run with it
+    if (c->use_persist || (c->fused_blocks && !c->prof)) return gb_md_segment(c, st, sites, 0, stream);   // its checks alone
     DeviceGuard g(c->device);
     cudaStream_t s = (cudaStream_t)stream;
     const size_t N = (size_t)c->N, M = (size_t)c->M;

@@ -60,3 +60,30 @@ def test_md_steps(pkg, sizes):
         runs.append(sim)
     for k in ("xyzq", "vel", "force", "R", "state"):
         assert torch.equal(getattr(runs[0], k), getattr(runs[1], k)), k
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_autotune_md_leaves_caps_it_does_not_use(pkg, persistent):
+    """A segment that runs in one launch reads no register caps: tuning on it
+    keeps those the context has, refuses what a segment refuses, and moves no
+    state; with profiling on the passes run one by one and are tuned."""
+    import torch
+    b = synth.random_batch([300, 180], seed=63)
+    sim = pkg.Simulation(b.atom_off, b.xyzq(), b.rad_screen(), pkg.default_params(rep_k=100.0, rep_sigma=2.5),
+                         sites=b.site_tables(), pH=b.pH, E=b.E, seed=9, mc_every=5)
+    sim.ctx.set_persistent(persistent)
+    x = sim.xyzq.clone()
+    for caps in ((4, 3, 1), (1, 4, 4), (3, 1, 3)):
+        for p, c in enumerate(caps):
+            sim.ctx.set_reg_cap(c, p)
+        assert sim.ctx.autotune_md(sim.st, sim.sites, 10) == caps
+    assert sim.step == 0 and torch.equal(sim.xyzq, x)
+    state, sim.st.state = sim.st.state, None
+    with pytest.raises(pkg.GBError):
+        sim.ctx.autotune_md(sim.st, sim.sites, 10)
+    sim.st.state = state
+    if not persistent:
+        sim.ctx.set_profiling(True)
+        assert all(c in (1, 3, 4) for c in sim.ctx.autotune_md(sim.st, sim.sites, 10))
+    sim.sync()
+    assert torch.equal(sim.xyzq, x)
