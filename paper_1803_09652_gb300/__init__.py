@@ -659,6 +659,9 @@ def _make_fn():
             F, phi = fctx.saved_tensors
             g_atom = g.to(torch.float64)
             if fctx.counts is not None:
+                # the counts belong to the stream of the context's first call, and
+                # this node may be the last to hold them
+                fctx.counts.record_stream(torch.cuda.current_stream(F.device))
                 g_atom = torch.repeat_interleave(g_atom, fctx.counts, output_size=F.shape[0])
             grad = torch.cat([F * -g_atom[:, None], (phi * g_atom)[:, None]], 1).float()
             return grad, None, None
