@@ -20,10 +20,10 @@
  *    errors are reported synchronously; gb_last_error() has the message.
  *    Errors detected on the device set a device error word that
  *    gb_sync_status() reads and clears (the first one recorded is kept):
- *    GB_ERR_NONFINITE for a non-finite coordinate, charge or Born radius,
- *    two atoms of a replica at the same position (coincident), or an atom so
- *    far from its neighbours in the chain that FP32 cannot hold the squared
- *    distance; GB_ERR_TIMEOUT
+ *    GB_ERR_NONFINITE for a non-finite coordinate, charge or Born radius, a
+ *    coordinate of 5e18 A or more (FP32 cannot hold squared distances much
+ *    past that), or two atoms of a replica at the same position (coincident);
+ *    GB_ERR_TIMEOUT
  *    for a bounded wait that gave up; GB_ERR_INVALID_ARG for a site table
  *    that fails the checks listed at gb_sites.
  *  - Per-atom layouts:

@@ -40,16 +40,22 @@ __device__ __forceinline__ float ghost_x(int local) { return 1.0e7f + 16.0f * (f
 
 __device__ __forceinline__ float shfl(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
+// No squared distance between coordinates below this overflows (12 COORD_MAX^2 <
+// FLT_MAX).  One that did would pass for infinitely far in the forms of 1/r^2 and
+// leave its atoms without an R dE/dR; only a run that has blown up gets here.
+constexpr float COORD_MAX = 5.0e18f;
+
 // Bounding box of one 32-atom tile, reduced over the warp (every lane calls
 // it; lanes without an atom pass valid = false): lo.xyz with the largest
 // a = rho - offset, hi.xyz with the largest screened radius s, stored by
 // lane 0 at boxes[2t], boxes[2t + 1].
-// Also the finiteness check of the evaluation's input: a lane whose atom has a
-// non-finite coordinate or charge records GB_ERR_NONFINITE (err nullable; the
-// int64 fixed-point sums would otherwise turn NaN into a silent zero).
+// Also the check of the evaluation's input: a lane whose atom has a coordinate
+// beyond COORD_MAX or not finite, or a charge that is not finite, records
+// GB_ERR_NONFINITE (err nullable; the int64 fixed-point sums would otherwise turn
+// NaN into a silent zero).
 __device__ __forceinline__ void tile_box_store(float4* boxes, int64_t t, bool valid, float x, float y, float z,
                                                float a, float s, float q, int* err) {
-    if (valid && err && !(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(q)))
+    if (valid && err && !(fabsf(x) < COORD_MAX && fabsf(y) < COORD_MAX && fabsf(z) < COORD_MAX && isfinite(q)))
         atomicCAS(err, 0, GB_ERR_NONFINITE);
     float x0 = valid ? x : INFINITY, y0 = valid ? y : INFINITY, z0 = valid ? z : INFINITY;
     float x1 = valid ? x : -INFINITY, y1 = valid ? y : -INFINITY, z1 = valid ? z : -INFINITY;

@@ -48,8 +48,8 @@ __device__ __forceinline__ int round_task(const PairArgs& A, int r, int K, int J
     float4 ih;
     const float4 il = row_box_lo(A, t0, K, nb, &ih);
     const BoxPair b = box_pair(il, ih, __ldcg(&A.boxes[2 * (t0 + J)]), __ldcg(&A.boxes[2 * (t0 + J) + 1]));
-    const int tier = row_tier<P, FLAGS>(A, b);
-    if (tier > 0 && J >= 2 * K + 2) {
+    const int tier = J < 2 * K + 2 ? 0 : row_tier<P, FLAGS>(A, b);
+    if (tier > 0) {
         run_far<P, FLAGS, 1>(tier, A, r, 64 * K, J, 1u, slot);
         return 0;
     }

@@ -1582,13 +1582,7 @@ template <class P, int FLAGS>
 __device__ __forceinline__ int row_tier(const PairArgs& A, const BoxPair& b) {
     if (P::RADIUS_CUT) {
         const float as = b.amax + b.smax, s2 = b.smax * b.smax;
-        if (b.rmin2 < as * as || s2 > GB_POLY_YFAR * b.rmin2) {
-            // atoms so far from their neighbours that r^2 overflows (a run that has
-            // blown up): 1/r^2 = 0 would pass for infinitely far, and the energy
-            // pass cannot give them an R dE/dR
-            if (!P::CHAIN && isinf(b.rmax2) && A.err) atomicCAS(A.err, 0, GB_ERR_NONFINITE);
-            return 0;
-        }
+        if (b.rmin2 < as * as || s2 > GB_POLY_YFAR * b.rmin2) return 0;
         const float y3 = P::CHAIN ? GB_Y_H3 : GB_Y_G3, y2 = P::CHAIN ? GB_Y_H2 : GB_Y_G2;
         return s2 <= y2 * b.rmin2 ? 3 : (s2 <= y3 * b.rmin2 ? 2 : 1);
     }

@@ -1,8 +1,6 @@
-"""Finite coordinates so far apart that the square of a distance overflows: an
-atom whose neighbours in the same 64 x 32 block are that far is reported as
-non-finite (distances of 1e19 A and more only come from a run that has blown
-up), without and with cutoffs, and the context evaluates valid input
-afterwards."""
+"""Finite coordinates so far apart that the square of a distance overflows (only
+a run that has blown up has them) are reported as non-finite, without and with
+cutoffs, and the context evaluates valid input afterwards."""
 import numpy as np
 import pytest
 
@@ -41,3 +39,17 @@ def test_overflowing_distances_are_reported(pkg, n, atom, cut):
     ctx.sync_status()
     for k in good:
         assert torch.equal(again[k], good[k])
+
+
+@pytest.mark.parametrize("n,atom", [(96, 70), (1300, 700)])
+def test_far_coordinates_that_do_not_overflow_are_taken(pkg, n, atom):
+    import torch
+    rep = synth.make_replica(n, 7, [])
+    rep.xyz[atom, 0] = 4.0e18
+    xyzq, rad = to_dev(synth.Batch([rep], pH=np.zeros(1), E=np.zeros(1)), device())
+    ctx = pkg.Context([0, n])
+    out = ctx.energy_forces(xyzq, rad)
+    ctx.sync_status()
+    a = np.float32(rep.rho[atom]) - np.float32(0.09)
+    assert out["R"][atom].item() == pytest.approx(float(a), rel=1e-7)      # no neighbour descreens it
+    assert torch.all(out["F"][atom] == 0)
