@@ -138,11 +138,20 @@ void cut_replica(const gb_ctx* c, int r, int tpt, std::vector<int4>& out) {
 // Any order gives the same fixed-point sums.
 bool near_first(const int4& a, const int4& b) { return a.z - (a.y & ~3) < b.z - (b.y & ~3); }
 
+// Replicas that take 128 x 32 blocks come before those that do not.  With the tasks
+// of both interleaved an SM runs both sets of block forms at once, whose code is too
+// much for its instruction cache (inferred from the times: five replicas of 6,000 to
+// 12,000 atoms, line at 9,600, 821 us an MD step interleaved, 762 in this order, 771
+// in the other; 2,000 to 16,000 atoms 777, 721 and 728).
 int build_tasks_into(gb_ctx* c, int tpt, gbk::TaskList& out) {
     std::vector<int4> t;
     t.reserve((size_t)(2 * c->total_cols / tpt + 1));
-    for (int r = 0; r < c->M; ++r) cut_replica(c, r, tpt, t);
-    std::stable_sort(t.begin(), t.end(), near_first);
+    for (const bool small : {false, true}) {
+        const size_t first = t.size();
+        for (int r = 0; r < c->M; ++r)
+            if (small == (c->off_h[r + 1] - c->off_h[r] <= 32 * gbk::SMALL_TILES)) cut_replica(c, r, tpt, t);
+        std::stable_sort(t.begin() + first, t.end(), near_first);
+    }
     if (out.d_tasks) cudaFree(out.d_tasks);
     out.d_tasks = nullptr;
     out.n_tasks = (int)t.size();

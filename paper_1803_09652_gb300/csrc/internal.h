@@ -22,7 +22,7 @@ struct PairArgs {
     float tau_ke;              // (1/eps_in - 1/eps_out) k_e
     float ke_out, kappa;       // k_e / eps_out and the salt's inverse Debye length (EF_SALT)
     float kc;                  // k_e / eps_in
-    float en_a, en_b, en_g;    // distant energy blocks (EnergyWide): set_energy_factors
+    float en_a, en_b, en_g;    // blocks of EnergyW: set_energy_factors
     float salt_l2;             // log2(eps_in / eps_out)
     float rep_k, rep_sigma;    // soft repulsion (rep_k == 0: off)
     float rgbmax;              // Born-radius cutoff (EF_CUT kernels of the Born and chain passes)
@@ -39,12 +39,18 @@ struct PairArgs {
     int* err;                  // device error word (non-finite input, nullable)
 };
 
-// Replicas of up to this many 32-atom tiles (6400 atoms) run 64 x 32 blocks
-// only (walk_task in pairs_impl.cuh).  3 x 4999 atoms in salt water: 187 us a
-// force call with 64 x 32 blocks, 211 with 128 x 32; 16 x 4096 Born radii 148
-// against 183; 25,000-atom replicas the other way round (38.5 ms an MD step of
-// 48 with 128 x 32 blocks, 51 with the 64 x 32 ones before them).
-constexpr int SMALL_TILES = 200;
+// Replicas of up to this many 32-atom tiles (12,800 atoms) run 64 x 32 blocks
+// only (walk_task in pairs_impl.cuh).  A pair costs less in 128 x 32 blocks, but a
+// pass of them ends later: the line is where a GPU with few replicas breaks even.
+// us, 64 x 32 / 128 x 32, of an MD step (with soft repulsion) and of a force call:
+//   1 x 8000   162 / 184, 149 / 164      5 x 9000 to 4500   465 / 563, 452 / 539
+//   1 x 9700   213 / 239, 202 / 213      5 x 9700 to 1212   315 / 373, 303 / 343
+//   1 x 12000  297 / 318, 286 / 292      5 x 12000 to 6000  730 / 815, 728 / 788
+//   1 x 14000  386 / 402, 374 / 370      5 x 14000          1614 / 1572, -
+//   1 x 16000  467 / 487, 453 / 451      5 x 16000          2080 / 1988, -
+// Full batches break even earlier (force calls): 16 x 6700 1255 / 1297, 16 x 8192
+// 1824 / 1837, 16 x 9000 2177 / 2132, 16 x 10007 2628 / 2420, 8 x 12000 1896 / 1815.
+constexpr int SMALL_TILES = 400;
 
 // One warp task: replica, row pair and rows (4 P + 1, 2 or 3: atoms
 // 128P .. 128P+63, the 64 after them, or both), first tile J (atoms
