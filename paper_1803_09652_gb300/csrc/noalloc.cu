@@ -31,6 +31,17 @@ constexpr int static_tasks(int nb) {
     return t;
 }
 constexpr int kMaxTasks = static_tasks(kMaxAtoms / 32);
+// Molecules of up to this many tiles (3,840 atoms) have too few such tasks to fill
+// the GPU: every 64 x 32 block is one.  us a call, 237 atoms 79 -> 38, with both cutoffs
+// at 12 A 210 -> 91; 1000 atoms 83 -> 44 and 237 -> 110; 3840 without and with cutoffs
+// 74 and 134 (4000 atoms in runs of columns 95 and 273).
+constexpr int kBlockTaskTiles = 120;
+constexpr int static_blocks(int nb) {
+    int t = 0;
+    for (int c = nb; c > 0; c -= 4) t += c + (c > 2 ? c - 2 : 0);
+    return t;
+}
+static_assert(static_blocks(kBlockTaskTiles) <= kMaxTasks, "task list");
 
 constexpr size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -80,7 +91,7 @@ int scratch_for_current_device(cudaStream_t s, unsigned char** out) {
 }
 
 // Work list of one molecule: the columns of every row pair in runs of
-// kColsPerTask, one task each.  Also writes atom_off = {0, n}.
+// kColsPerTask, one task each, or every block.  Also writes atom_off = {0, n}.
 __global__ void k_static_tasks(int n, int nb, int n_tasks, int4* tasks, int64_t* atom_off, int* ctr) {
     gbk::pdl_enter();
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
@@ -93,6 +104,12 @@ __global__ void k_static_tasks(int n, int nb, int n_tasks, int4* tasks, int64_t*
     }
     if (w >= n_tasks) return;
     int t = w, PR = 0;
+    if (nb <= kBlockTaskTiles) {
+        int c = nb;
+        for (; t >= c + max(c - 2, 0); c -= 4, ++PR) t -= c + max(c - 2, 0);
+        tasks[w] = t < c ? make_int4(0, 4 * PR + 1, 4 * PR + t, 1) : make_int4(0, 4 * PR + 2, 4 * PR + 2 + t - c, 1);
+        return;
+    }
     for (int c = nb; c > 0; c -= 4, ++PR) {
         const int k = (c + kColsPerTask - 1) / kColsPerTask;
         if (t < k) break;
@@ -118,7 +135,7 @@ extern "C" int gb_energy_forces_static(int32_t n_atoms, const gb_params* params,
     if (rc) return rc;
     const int n = n_atoms;
     const int nb = (n + 31) / 32;
-    const int n_tasks = static_tasks(nb);
+    const int n_tasks = nb <= kBlockTaskTiles ? static_blocks(nb) : static_tasks(nb);
 
     gbk::u64* I_acc = (gbk::u64*)(base + kOffI);
     gbk::u64* dR_acc = (gbk::u64*)(base + kOffDR);

@@ -176,3 +176,34 @@ def test_one_launch_steps_with_salt(pkg, sizes):
         sim.ctx.set_profiling(prof)
         runs.append(sim.run(20).run(3))
     _equal(*runs)
+
+
+@pytest.mark.parametrize("field", [dict(rgbmax=12.0, cut=12.0), dict(rgbmax=9.0), dict(cut=25.0, kappa=0.125)])
+def test_cutoff_forces_do_not_depend_on_the_batch(pkg, field):
+    """Few blocks in the batch: every block in range is a task; many: runs of them."""
+    few, _ = _forces(pkg, [500, 1057, 33], field)
+    many, _ = _forces(pkg, [500, 1057, 33, 12000, 12000], field)
+    n = 500 + 1057 + 33
+    for k in few:
+        a, b = (few[k], many[k][:, :n]) if k == "F_fixed" else (few[k], many[k][:n])
+        assert np.array_equal(a, b), k
+
+
+@pytest.mark.parametrize("field", [{}, dict(rgbmax=12.0, cut=12.0)])
+@pytest.mark.parametrize("n", [1, 33, 65, 129, 3840, 3841])
+def test_static_entry_at_the_edges_of_its_task_lists(pkg, n, field):
+    """Every block a task up to 3840 atoms, runs of columns beyond.  Without tile boxes
+    a block may take another form than the context's; each is within its tolerance of
+    the oracle, so the two are within twice that."""
+    import torch
+    out, b = _forces(pkg, [n], field)
+    xyzq, rad = to_dev(b, device())
+    R, F = torch.empty(n, device=xyzq.device), torch.empty((n, 3), device=xyzq.device)
+    call = ctypes.CDLL(pkg.LIB_PATH).gb_energy_forces_static
+    call.argtypes = [ctypes.c_int32, ctypes.c_void_p] + [ctypes.c_void_p] * 8
+    params = pkg.default_params(**field)
+    assert call(n, ctypes.byref(params), xyzq.data_ptr(), rad.data_ptr(), R.data_ptr(), None, F.data_ptr(), None, None,
+                torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    assert np.max(np.abs(R.cpu().numpy() / out["R"] - 1)) < 2 * R_REL
+    assert np.max(np.abs(F.cpu().numpy() - out["F"])) < 2 * F_ABS
