@@ -358,8 +358,8 @@ int evaluate(gb_ctx* c, const float* xyzq, const float* rad, float* R_out, int f
     const gbk::AtomArgs aa = atom_args(c, xyzq, rad);
     if (build_boxes) GB_CHECK(c, gbk::launch_tile_boxes(pa, c->M, c->n_tiles32, s));
     if (c->list_ctr)
-        GB_CHECK(c, gbk::launch_block_list(pa, c->win_off, c->M, c->list_warps, c->list_b, c->list_e, c->list_ctr,
-                                           c->list_b ? 1 : 0, c->list_e ? 1 : 0, s));
+        GB_CHECK(c, gbk::launch_block_list(pa, c->win_off, c->M, c->list_warps, c->total_cols, c->list_b, c->list_e,
+                                           c->list_ctr, c->list_b ? 1 : 0, c->list_e ? 1 : 0, s));
     if (ev) GB_CHECK(c, mark(c, ev[0], s));
     GB_CHECK(c, pass(c, gbk::PASS_BORN, 0, pa, s));
     if (ev) GB_CHECK(c, mark(c, ev[1], s));
@@ -637,8 +637,8 @@ extern "C" int gb_born_radii(gb_ctx* c, const float* xyzq, const float* rad, flo
     const gbk::AtomArgs aa = atom_args(c, xyzq, rad);
     GB_CHECK(c, gbk::launch_tile_boxes(pa, c->M, c->n_tiles32, s));
     if (c->list_b)
-        GB_CHECK(c, gbk::launch_block_list(pa, c->win_off, c->M, c->list_warps, c->list_b, nullptr, c->list_ctr, 1, 0,
-                                           s));
+        GB_CHECK(c, gbk::launch_block_list(pa, c->win_off, c->M, c->list_warps, c->total_cols, c->list_b, nullptr,
+                                           c->list_ctr, 1, 0, s));
     GB_CHECK(c, pass(c, gbk::PASS_BORN, 0, pa, s));
     GB_CHECK(c, gbk::launch_born_finalize(aa, R_out, s));
     return GB_OK;

@@ -80,12 +80,12 @@ cudaError_t launch_pairs(int pass, int flags, const PairArgs& a, const TaskList&
 // (Born-radius cutoff, when want_b) and list_e (pair cutoff, when want_e),
 // each with room for both rows of every column of the batch; win_off [M+1] holds the first
 // list-building warp of each replica (ceil(nb/4) * ceil(nb/32) warps per
-// replica of nb tiles).  launch_pairs_list runs pass `pass` with EF_CUT over
+// replica of nb tiles), columns the batch's columns.  launch_pairs_list runs pass `pass` with EF_CUT over
 // a device-built task list whose length is ctr[0] (Born, chain) or ctr[1]
 // (energy), taking tasks from the queue head ctr[2 + pass].
 constexpr int LIST_CTRS = 5;
-cudaError_t launch_block_list(const PairArgs& a, const int* win_off, int M, int total_warps, int4* list_b,
-                              int4* list_e, int* ctr, int want_b, int want_e, cudaStream_t s);
+cudaError_t launch_block_list(const PairArgs& a, const int* win_off, int M, int total_warps, int64_t columns,
+                              int4* list_b, int4* list_e, int* ctr, int want_b, int want_e, cudaStream_t s);
 cudaError_t launch_pairs_list(int pass, int flags, const PairArgs& a, const int4* list, int* ctr, int cap,
                               int warps_per_block, cudaStream_t s);
 

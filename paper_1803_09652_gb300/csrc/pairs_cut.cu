@@ -4,7 +4,7 @@
 // evaluation (k_tile_boxes, or k_md_step in the MD driver).  One warp covers
 // 32 consecutive columns J0 .. J0+31 of a row pair: lane l classifies the two
 // blocks of column J0 + l with cut_class, a ballot per row gives the warp the
-// bits of the blocks in range, and every run of them (cut at RUN) becomes one
+// bits of the blocks in range, and every run of them (cut at `run`) becomes one
 // task of a compacted list, placed with one atomic per row and warp.  Two lists: the Born-radius cutoff's (Born and chain
 // passes) and the pair cutoff's (energy pass).  The passes then take the
 // tasks from a queue (k_pairs_dyn): blocks out of range cost nothing, and
@@ -19,7 +19,14 @@ namespace gbk {
 
 namespace {
 
-constexpr int RUN = 4;           // blocks per task at most (100,000 atoms, 12 A: 1.64 ms; 8: 1.73; at 25 A 3.97 and 3.94)
+// Blocks per task at most.  Large batches: 4 (100,000 atoms, 12 A: 1.64 ms; 8: 1.73;
+// at 25 A 3.97 and 3.94).  Where the whole batch has at most 256 blocks an SM, in range or
+// not, every block is a task, so that no warp evaluates four with their close pairs
+// while others have none.  us a force call at 12 A with runs of 4 / single blocks: 1 x 1024
+// 233 / 107, 8 x 2048 313 / 205, 1 x 10007 286 / 180, 4 x 5000 337 / 267; MD step of 1000 x 64
+// 181 / 140.  (Lines at 16 and 64 blocks an SM leave the last two, three as they were;
+// 16 x 4096 atoms, 430 an SM: 683 with runs of 4.)
+constexpr int RUN = 4, FEW_BLOCKS = 152 * 256;
 
 __global__ void k_list_reset(int* ctr) {
     pdl_enter();
@@ -27,10 +34,10 @@ __global__ void k_list_reset(int* ctr) {
 }
 
 // Appends the runs of set bits of m (lanes = columns J0 ..) to a list.
-__device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int row, int J0, int4* list, int* counter) {
+__device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int row, int J0, int run, int4* list, int* counter) {
     const bool on = (m >> lane) & 1u;
     const bool prev = lane > 0 && ((m >> (lane - 1)) & 1u);
-    const bool start = on && (!prev || (lane & (RUN - 1)) == 0);
+    const bool start = on && (!prev || (lane & (run - 1)) == 0);
     const unsigned sm = __ballot_sync(0xffffffffu, start);
     if (!sm) return;
     int base = 0;
@@ -39,7 +46,7 @@ __device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int row, 
     if (start) {
         const unsigned rest = ~(m >> lane);          // the run ends at the first zero
         int len = rest ? __ffs(rest) - 1 : 32 - lane;
-        len = min(len, RUN - (lane & (RUN - 1)));
+        len = min(len, run - (lane & (run - 1)));
         list[base + __popc(sm & ((1u << lane) - 1u))] = make_int4(r, row, J0 + lane, len);
     }
 }
@@ -47,7 +54,7 @@ __device__ __forceinline__ void emit_runs(unsigned m, int lane, int r, int row, 
 // win_off[r]: first warp of replica r; a replica has ceil(nb/4) row pairs of
 // ceil(nb/32) warps each (warps past the row's last column exit).
 __global__ void k_block_list(PairArgs A, const int* __restrict__ win_off, int M, int total, int4* list_b,
-                             int4* list_e, int* ctr, int want_b, int want_e) {
+                             int4* list_e, int* ctr, int want_b, int want_e, int run) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -85,8 +92,8 @@ __global__ void k_block_list(PairArgs A, const int* __restrict__ win_off, int M,
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        if (want_b) emit_runs(__ballot_sync(0xffffffffu, in_b[h]), lane, r, 4 * PR + 1 + h, J0, list_b, &ctr[0]);
-        if (want_e) emit_runs(__ballot_sync(0xffffffffu, in_e[h]), lane, r, 4 * PR + 1 + h, J0, list_e, &ctr[1]);
+        if (want_b) emit_runs(__ballot_sync(0xffffffffu, in_b[h]), lane, r, 4 * PR + 1 + h, J0, run, list_b, &ctr[0]);
+        if (want_e) emit_runs(__ballot_sync(0xffffffffu, in_e[h]), lane, r, 4 * PR + 1 + h, J0, run, list_e, &ctr[1]);
     }
 }
 
@@ -155,12 +162,12 @@ cudaError_t energy_dyn(int flags, const PairArgs& a, const int4* list, int* ctr,
 
 }  // namespace
 
-cudaError_t launch_block_list(const PairArgs& a, const int* win_off, int M, int total_warps, int4* list_b,
-                              int4* list_e, int* ctr, int want_b, int want_e, cudaStream_t s) {
+cudaError_t launch_block_list(const PairArgs& a, const int* win_off, int M, int total_warps, int64_t columns,
+                              int4* list_b, int4* list_e, int* ctr, int want_b, int want_e, cudaStream_t s) {
     cudaError_t e = launch_pdl(k_list_reset, dim3(1), dim3(32), 0, s, ctr);
     if (e != cudaSuccess || total_warps == 0) return e;
     return launch_pdl(k_block_list, dim3((total_warps + 7) / 8), dim3(256), 0, s, a, win_off, M, total_warps,
-                      list_b, list_e, ctr, want_b, want_e);
+                      list_b, list_e, ctr, want_b, want_e, 2 * columns <= FEW_BLOCKS ? 1 : RUN);
 }
 
 cudaError_t launch_pairs_list(int pass, int flags, const PairArgs& a, const int4* list, int* ctr, int cap, int wpb,
