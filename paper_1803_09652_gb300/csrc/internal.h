@@ -303,9 +303,8 @@ struct PersistArgs {
     int* err;
     unsigned spin_limit;       // polls before a dependency wait gives up (GB_ERR_TIMEOUT)
 };
-size_t persist_smem();
-cudaError_t persist_occupancy(int rep, int* blocks_per_sm);
-cudaError_t launch_persist(const PersistArgs& a, int rep, int grid, cudaStream_t s);
+cudaError_t persist_occupancy(int rep, bool small, int* blocks_per_sm);
+cudaError_t launch_persist(const PersistArgs& a, int rep, bool small, int grid, cudaStream_t s);
 
 // Small batches in one launch (fused.cu).
 constexpr int FUSED_WARPS = 8;     // warps of a thread block

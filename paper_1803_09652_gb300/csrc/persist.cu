@@ -55,8 +55,13 @@ __device__ __forceinline__ bool wait_count(const unsigned* ctr, unsigned target,
     return ok != 0;
 }
 
-template <int REP>
-__global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(const __grid_constant__ PersistArgs P) {
+// Four blocks an SM at 128 registers: at 80 (six blocks, of which shared memory
+// holds five) the pair code spilled 700 to 980 bytes a thread.  us an MD step with
+// 80 / 96 / 128 registers: 8 x 2048 176 / 164 / 153, 16 x 4096 801 / 746 / 698, 4 x 300
+// 70 / 64 / 55, 8 x 25000 8160 / 7830 / 7780.  SMALL as in walk_task: 158 and 720 us
+// for the first two without it.
+template <int REP, bool SMALL>
+__global__ void __launch_bounds__(PERSIST_THREADS, 4) k_md_persist(const __grid_constant__ PersistArgs P) {
     constexpr int EFL = REP ? EF_REP : 0;
     const int lane = threadIdx.x & 31;
     const int slot = (threadIdx.x >> 5) * PERSIST_SMEM;
@@ -93,16 +98,16 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(const __grid_
         if (!ok) break;
         switch (p) {
             case 0: tile_halfsteps(P, r, u, lane, s > 0, s < P.nsteps, step0 + (u64)s + 1); break;
-            case 1: walk_task<Born, 0>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
+            case 1: walk_task<Born, 0, SMALL>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
             case 2: {
                 const int64_t base = P.pa.atom_off[r];
                 const int i = 32 * u + lane;
                 if (i < (int)(P.pa.atom_off[r + 1] - base)) born_finalize_atom(P.aa, base + i, P.R_out);
                 break;
             }
-            case 3: walk_task<EnergyF<EFL>, EFL>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
+            case 3: walk_task<EnergyF<EFL>, EFL, SMALL>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
             case 4: atoms_chain_bonds(P, r, u, lane); break;
-            default: walk_task<Chain, 0>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
+            default: walk_task<Chain, 0, SMALL>(P.pa, P.tasks[P.task_off[r] + u], slot, lane); break;
         }
         __threadfence();
         __syncwarp();
@@ -110,21 +115,25 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 6) k_md_persist(const __grid_
     }
 }
 
-size_t persist_smem() { return (size_t)(PERSIST_THREADS / 32) * PERSIST_SMEM; }
+namespace {
+constexpr size_t PERSIST_BLOCK_SMEM = (PERSIST_THREADS / 32) * PERSIST_SMEM;
+typedef void (*PersistKernel)(PersistArgs);
+PersistKernel persist_kernel(int rep, bool small) {
+    if (small) return rep ? k_md_persist<1, true> : k_md_persist<0, true>;
+    return rep ? k_md_persist<1, false> : k_md_persist<0, false>;
+}
+}  // namespace
 
-cudaError_t persist_occupancy(int rep, int* blocks_per_sm) {
-    const size_t smem = persist_smem();
-    if (rep) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_md_persist<1>, PERSIST_THREADS, smem);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_md_persist<0>, PERSIST_THREADS, smem);
+cudaError_t persist_occupancy(int rep, bool small, int* blocks_per_sm) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, persist_kernel(rep, small), PERSIST_THREADS,
+                                                         PERSIST_BLOCK_SMEM);
 }
 
-cudaError_t launch_persist(const PersistArgs& a, int rep, int grid, cudaStream_t s) {
+cudaError_t launch_persist(const PersistArgs& a, int rep, bool small, int grid, cudaStream_t s) {
     // queue head and the per-(phase, replica) completion counters start at zero
     cudaError_t e = cudaMemsetAsync(a.head, 0, sizeof(unsigned) * (1 + 6 * (size_t)a.M), s);
     if (e != cudaSuccess) return e;
-    const size_t smem = persist_smem();
-    if (rep) k_md_persist<1><<<grid, PERSIST_THREADS, smem, s>>>(a);
-    else k_md_persist<0><<<grid, PERSIST_THREADS, smem, s>>>(a);
+    persist_kernel(rep, small)<<<grid, PERSIST_THREADS, PERSIST_BLOCK_SMEM, s>>>(a);
     return cudaGetLastError();
 }
 
