@@ -202,8 +202,7 @@ __device__ __forceinline__ f2 hct_cut2(f2 r, f2 rinv, f2 a, f2 s, float rc, floa
 //   dB/dr = -dL/L^2 + dU/U'^2 + (1 + s^2/r^2)/4 (1/U'^2 - 1/L^2)
 //           + w/2 (dL/L^3 - dU/U'^3) - ln(L/U') / (2 r^2) + (dL/L - dU/U') / (2r)
 // (0 when L >= U'), plus 2 dL/L^2 when engulfed with L < rc.
-// (out of line: the chain pass's straddle code would not fit the instruction
-// cache with it inlined into every block mode)
+// (out of line: only overlapping pairs near the cutoff take it)
 static __device__ __noinline__ f2 hct_cut_fr2(f2 r, f2 rinv, f2 a, f2 s, float rc) {
     const f2 U = add2(r, s);
     const bool cx = U.x > rc, cy = U.y > rc;
@@ -790,7 +789,7 @@ __device__ __forceinline__ f2 screen_r2(f2 r2, Mask m, Ring g, unsigned bit, uns
     return make_float2(kx && m.x ? r2.x : FAR_R2, ky && m.y ? r2.y : FAR_R2);
 }
 
-// The staged tile of a warp: j atoms (twice, see stage()), what close pairs
+// The staged tile of a warp: j atoms (twice, see walk_far), what close pairs
 // need of both sides, their j sums and their queue.
 constexpr int CLOSE_CAP = 512;
 template <class W>
@@ -1725,9 +1724,8 @@ __device__ __forceinline__ void walk_task(const PairArgs& A, const int4 t, int s
 
 
 // --- the pair-pass kernel --------------------------------------------------------
-// One warp per task.  MINB = 1 leaves the register count to the compiler;
-// MINB = 3 or 4 caps it so that three or four 256-thread blocks fit on an SM
-// (more warps, some spills).
+// One warp per task.  MINB caps the registers so that two, three or four
+// 256-thread blocks fit on an SM (128, 80, 64 a thread: more warps, more spills).
 template <class P, int FLAGS, int MINB, bool SMALL>
 __global__ void __launch_bounds__(256, MINB) k_pairs(const __grid_constant__ PairArgs A, const int4* __restrict__ tasks, int n_tasks) {
     pdl_enter();
